@@ -65,6 +65,8 @@ static ytn_status upload(ytn_plan_t *p) {
   size_t o_csj;
   put_table(buf, p->cs_jobs, o_csj);
   put_table(buf, p->tr_contrib, o_trc);
+  size_t o_trk;
+  put_table(buf, p->tr_chunks, o_trk);
   size_t o_vdp, o_vdc;
   put_table(buf, p->vd_pieces, o_vdp);
   put_table(buf, p->vd_chunks, o_vdc);
@@ -97,6 +99,7 @@ static ytn_status upload(ytn_plan_t *p) {
   p->d_tr_out = reinterpret_cast<const TraceOut *>(d + o_tro);
   p->d_cs_jobs = reinterpret_cast<const CScatterJob *>(d + o_csj);
   p->d_tr_contrib = reinterpret_cast<const TraceContrib *>(d + o_trc);
+  p->d_tr_chunks = reinterpret_cast<const TraceChunk *>(d + o_trk);
   p->d_vd_pieces = reinterpret_cast<const VdotPiece *>(d + o_vdp);
   p->d_vd_chunks = reinterpret_cast<const VdotChunk *>(d + o_vdc);
   p->d_sp_ops = reinterpret_cast<const SplitOperand *>(d + o_spo);
@@ -1104,7 +1107,7 @@ static ytn_status run_move(ytn_plan_t *p, Kind k, const double *a, double *out, 
     return cuda_fail(e, "memset output");
   PhaseTimer t(p->ctx, YTN_PHASE_MOVE, st);
   if (k == Kind::Trace) {
-    if ((e = launch_trace(p->d_tr_out, (int64_t)p->tr_out.size(), p->d_tr_contrib, a, out, st)) != cudaSuccess)
+    if ((e = launch_trace(p->d_tr_chunks, (int64_t)p->tr_chunks.size(), p->d_tr_out, p->d_tr_contrib, a, out, st)) != cudaSuccess)
       return cuda_fail(e, "trace");
     return YTN_OK;
   }

@@ -247,40 +247,85 @@ __global__ void __launch_bounds__(kThreads) zero_flagged_kernel(const SectorDev 
   }
 }
 
-// Trace: thread per output element; contributing blocks and diagonal elements
-// are summed in a fixed order.
-__global__ void __launch_bounds__(128) trace_kernel(const TraceOut *__restrict__ outs,
-                                                    const TraceContrib *__restrict__ contribs,
-                                                    const double *__restrict__ src,
-                                                    double *__restrict__ dst) {
-  const TraceOut o = outs[blockIdx.x];
-  for (int e = threadIdx.x; e < o.nrest; e += blockDim.x) {
-    int idx[kMaxCopyDims];
-    int r = e;
-    for (int i = o.nrd - 1; i >= 0; i--) {
-      idx[i] = r % o.rext[i];
-      r /= o.rext[i];
-    }
-    double sum = 0.0;
-    for (int c = o.first; c < o.first + o.ncontrib; c++) {
-      const TraceContrib &tc = contribs[c];
-      int64_t base = tc.src_off;
-      for (int i = 0; i < o.nrd; i++) base += (int64_t)idx[i] * tc.rstr[i];
-      int P = 1;
-      for (int k = 0; k < tc.ndiag; k++) P *= tc.dext[k];
-      for (int d = 0; d < P; d++) {
-        int rem = d;
-        int64_t off = base;
-        for (int k = tc.ndiag - 1; k >= 0; k--) {
-          const int dk = rem % tc.dext[k];
-          rem /= tc.dext[k];
-          off += (int64_t)dk * tc.dstr[k];
+// Trace: a CTA takes kTraceElems elements of one output block. Its threads are
+// `wide` lanes over the elements (32, or the power of two that holds a smaller
+// block) times kTraceThreads / wide workers, each summing an equal contiguous share
+// of the block's terms (the diagonal elements of its contributing blocks in order);
+// the workers' sums are added in a fixed order, so repeated calls give the same
+// bits. Latency-bound: the terms are single elements far apart in memory, so the
+// time is a thread's chain of loads, eight in flight; spreading the terms over 512
+// threads took the D = 16 environment's partial trace (61 output blocks, about 256
+// terms each) from 769 us (thread per output element, one CTA per block) to 24 us.
+constexpr int kTraceThreads = 512;
+
+__global__ void __launch_bounds__(kTraceThreads) trace_kernel(const TraceChunk *__restrict__ chunks,
+                                                              const TraceOut *__restrict__ outs,
+                                                              const TraceContrib *__restrict__ contribs,
+                                                              const double *__restrict__ src,
+                                                              double *__restrict__ dst) {
+  __shared__ double part[kTraceThreads];
+  const TraceChunk ch = chunks[blockIdx.x];
+  const TraceOut &o = outs[ch.out];
+  const int ne = min(kTraceElems, o.nrest - ch.e0);
+  int wide = kTraceElems;
+  while (wide / 2 >= ne) wide >>= 1;
+  const int lane = threadIdx.x & (wide - 1), worker = threadIdx.x / wide, nworkers = kTraceThreads / wide;
+  double sum = 0.0;
+  if (lane < ne) {
+    const int64_t nterms = o.nterms;
+    const int64_t t0 = nterms * worker / nworkers, t1 = nterms * (worker + 1) / nworkers;
+    if (t0 < t1) {
+      int idx[kMaxCopyDims];
+      int r = ch.e0 + lane;
+#pragma unroll
+      for (int i = kMaxCopyDims - 1; i >= 0; i--)
+        if (i < o.nrd) {
+          idx[i] = r % o.rext[i];
+          r /= o.rext[i];
         }
-        sum += src[off];
+      // first contribution: the last one whose terms start at or before t0
+      int lo = 0, hi = o.ncontrib - 1;
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (contribs[o.first + mid].term0 <= t0) lo = mid;
+        else hi = mid - 1;
+      }
+      int64_t t = t0;
+      for (int c = lo; t < t1; c++) {
+        const TraceContrib &tc = contribs[o.first + c];
+        const int64_t end = c + 1 < o.ncontrib ? min(t1, contribs[o.first + c + 1].term0) : t1;
+        int64_t base = tc.src_off;
+#pragma unroll
+        for (int i = 0; i < kMaxCopyDims; i++)
+          if (i < o.nrd) base += (int64_t)idx[i] * tc.rstr[i];
+        if (tc.ndiag == 1) {   // one pair: the terms lie a constant stride apart
+          const int64_t st = tc.dstr[0];
+          const double *q = src + base + (t - tc.term0) * st;
+#pragma unroll 8
+          for (; t < end; t++, q += st) sum += *q;
+        } else {
+          for (; t < end; t++) {
+            int rem = (int)(t - tc.term0);
+            int64_t off = base;
+            for (int k = tc.ndiag - 1; k >= 0; k--) {
+              const int dk = rem % tc.dext[k];
+              rem /= tc.dext[k];
+              off += (int64_t)dk * tc.dstr[k];
+            }
+            sum += src[off];
+          }
+        }
       }
     }
-    dst[o.dst_off + e] = sum;
   }
+  part[threadIdx.x] = sum;
+  __syncthreads();
+  // the workers' sums, halved in a fixed tree
+  for (int h = nworkers / 2; h > 0; h >>= 1) {
+    if (worker < h) part[worker * wide + lane] += part[(worker + h) * wide + lane];
+    __syncthreads();
+  }
+  if (worker == 0 && lane < ne) dst[o.dst_off + ch.e0 + lane] = part[lane];
 }
 
 // Scatter-combine of a complex product: the doubled real C_q holds the four
@@ -327,11 +372,11 @@ cudaError_t launch_copy(const CopyJob *jobs, const CopyItem *items, int64_t nite
   return cudaGetLastError();
 }
 
-cudaError_t launch_trace(const TraceOut *outs, int64_t nout, const TraceContrib *contribs,
-                         const double *src, double *dst, cudaStream_t stream) {
-  if (nout <= 0) return cudaSuccess;
-  if (nout > INT32_MAX) return cudaErrorInvalidValue;
-  trace_kernel<<<(unsigned)nout, 128, 0, stream>>>(outs, contribs, src, dst);
+cudaError_t launch_trace(const TraceChunk *chunks, int64_t nchunks, const TraceOut *outs,
+                         const TraceContrib *contribs, const double *src, double *dst, cudaStream_t stream) {
+  if (nchunks <= 0) return cudaSuccess;
+  if (nchunks > INT32_MAX) return cudaErrorInvalidValue;
+  trace_kernel<<<(unsigned)nchunks, kTraceThreads, 0, stream>>>(chunks, outs, contribs, src, dst);
   return cudaGetLastError();
 }
 

@@ -13,9 +13,9 @@ namespace ytn {
 cudaError_t launch_copy(const CopyJob *jobs, const CopyItem *items, int64_t nitems, const double *src,
                         double *dst, cudaStream_t stream, int max_nd = kMaxCopyDims);
 
-// Trace: one CTA per output block.
-cudaError_t launch_trace(const TraceOut *outs, int64_t nout, const TraceContrib *contribs,
-                         const double *src, double *dst, cudaStream_t stream);
+// Trace: one CTA per chunk of an output block.
+cudaError_t launch_trace(const TraceChunk *chunks, int64_t nchunks, const TraceOut *outs,
+                         const TraceContrib *contribs, const double *src, double *dst, cudaStream_t stream);
 
 // Scalar product <A, B> over the planned common elements (FP64, deterministic):
 // one partial per chunk into `partials`, then their fixed-order sum into out[0].

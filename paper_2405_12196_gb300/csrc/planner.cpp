@@ -1789,6 +1789,7 @@ ytn_status plan_trace(ytn_plan_t *p, const Tensor &A, int naxes, const int *ax1_
   finalize_out(C, sorted, off_of_id);
   p->tr_out.clear();
   p->tr_contrib.clear();
+  p->tr_chunks.clear();
   int64_t id = 0;
   for (auto &kv : contrib) {
     TraceOut to{};
@@ -1810,8 +1811,11 @@ ytn_status plan_trace(ytn_plan_t *p, const Tensor &A, int naxes, const int *ax1_
       to.nrest *= 2;
       to.rext[to.nrd++] = 2;
     }
+    int64_t terms = 0;   // diagonal elements of the contributions before this one
     for (int64_t b : kv.second) {
       TraceContrib tc{};
+      tc.term0 = terms;
+      terms += sub_elems(A, b, ax1);
       tc.src_off = w * A.off[b];
       auto st = block_strides(A, b);
       for (size_t i = 0; i < rest.size(); i++) tc.rstr[i] = (int32_t)(w * st[rest[i]]);
@@ -1823,6 +1827,8 @@ ytn_status plan_trace(ytn_plan_t *p, const Tensor &A, int naxes, const int *ax1_
       }
       p->tr_contrib.push_back(tc);
     }
+    to.nterms = terms;
+    for (int64_t e = 0; e < to.nrest; e += kTraceElems) p->tr_chunks.push_back({(int32_t)p->tr_out.size(), (int32_t)e});
     p->tr_out.push_back(to);
     id++;
   }
@@ -1883,8 +1889,22 @@ ytn_status plan_vdot(ytn_plan_t *p, const Tensor &A, const Tensor &B, std::strin
     if (ka < kb) { i++; continue; }
     if (kb < ka) { j++; continue; }
     const int64_t n = A.elems(i), nd = cw * n;
-    for (int64_t e = 0; e < nd; e += kVdotPiece)
-      p->vd_pieces.push_back({cw * A.off[i] + e, cw * B.off[j] + e, (int32_t)std::min<int64_t>(kVdotPiece, nd - e), 0});
+    // a block that follows the previous common one in both tensors extends its run
+    // (tensors of the same structure are one run, whatever their block sizes)
+    int64_t e = 0;
+    while (e < nd) {
+      VdotPiece *last = p->vd_pieces.empty() ? nullptr : &p->vd_pieces.back();
+      const int64_t ao = cw * A.off[i] + e, bo = cw * B.off[j] + e;
+      if (last && last->len < kVdotPiece && last->a_off + last->len == ao && last->b_off + last->len == bo) {
+        const int32_t m = (int32_t)std::min<int64_t>(kVdotPiece - last->len, nd - e);
+        last->len += m;
+        e += m;
+      } else {
+        const int32_t m = (int32_t)std::min<int64_t>(kVdotPiece, nd - e);
+        p->vd_pieces.push_back({ao, bo, m, 0});
+        e += m;
+      }
+    }
     common += n;
     i++;
     j++;

@@ -86,9 +86,15 @@ struct GemmTile {
   int32_t size;     // tile edge: 64, or 32 for small sectors
 };
 
-// Trace: one output block, fed by ncontrib contributing input blocks.
+// Trace: one output block, fed by ncontrib contributing input blocks with nterms
+// diagonal elements in all; a CTA takes kTraceElems of its elements (TraceChunk).
+constexpr int kTraceElems = 32;
+struct TraceChunk {
+  int32_t out, e0;
+};
 struct TraceOut {
   int64_t dst_off;
+  int64_t nterms;
   int32_t nrest;          // elements of the output block
   int32_t nrd;            // rest dims
   int32_t first, ncontrib;
@@ -96,6 +102,7 @@ struct TraceOut {
 };
 struct TraceContrib {
   int64_t src_off;
+  int64_t term0;          // diagonal elements of the output's contributions before this one
   int32_t ndiag;          // paired dims
   int32_t pad;
   int32_t rstr[kMaxCopyDims];   // input strides of the rest dims
@@ -386,6 +393,7 @@ struct ytn_plan_s {
   std::vector<ytn::TraceOut> tr_out;
   std::vector<ytn::CScatterJob> cs_jobs;   // complex tensordot: the scatter-combine
   std::vector<ytn::TraceContrib> tr_contrib;
+  std::vector<ytn::TraceChunk> tr_chunks;
   std::vector<ytn::VdotPiece> vd_pieces;
   std::vector<ytn::VdotChunk> vd_chunks;
 
@@ -399,6 +407,7 @@ struct ytn_plan_s {
   const ytn::TraceOut *d_tr_out = nullptr;
   const ytn::CScatterJob *d_cs_jobs = nullptr;
   const ytn::TraceContrib *d_tr_contrib = nullptr;
+  const ytn::TraceChunk *d_tr_chunks = nullptr;
   const ytn::VdotPiece *d_vd_pieces = nullptr;
   const ytn::VdotChunk *d_vd_chunks = nullptr;
 
