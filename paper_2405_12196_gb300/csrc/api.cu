@@ -64,6 +64,8 @@ static ytn_status upload(ytn_plan_t *p) {
   put_table(buf, p->tr_out, o_tro);
   size_t o_csj;
   put_table(buf, p->cs_jobs, o_csj);
+  size_t o_csk;
+  put_table(buf, p->cs_chunks, o_csk);
   put_table(buf, p->tr_contrib, o_trc);
   size_t o_trk;
   put_table(buf, p->tr_chunks, o_trk);
@@ -98,6 +100,7 @@ static ytn_status upload(ytn_plan_t *p) {
   p->d_tiles = reinterpret_cast<const GemmTile *>(d + o_tiles);
   p->d_tr_out = reinterpret_cast<const TraceOut *>(d + o_tro);
   p->d_cs_jobs = reinterpret_cast<const CScatterJob *>(d + o_csj);
+  p->d_cs_chunks = reinterpret_cast<const CScatterChunk *>(d + o_csk);
   p->d_tr_contrib = reinterpret_cast<const TraceContrib *>(d + o_trc);
   p->d_tr_chunks = reinterpret_cast<const TraceChunk *>(d + o_trk);
   p->d_vd_pieces = reinterpret_cast<const VdotPiece *>(d + o_vdp);
@@ -857,7 +860,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
   {
     PhaseTimer t(p->ctx, YTN_PHASE_SCATTER, st);
     if (p->ca * p->cb > 1)
-      e = launch_cscatter(p->d_cs_jobs, (int64_t)p->cs_jobs.size(), wc, c, st);
+      e = launch_cscatter(p->d_cs_jobs, p->d_cs_chunks, (int64_t)p->cs_chunks.size(), wc, c, st);
     else
       e = copy_range(p, p->items_c_begin, p->items_c_end, wc, c, st);
   }

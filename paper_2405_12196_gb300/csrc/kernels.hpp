@@ -49,9 +49,9 @@ cudaError_t configure_split_gemm();
 cudaError_t configure_split_blocks();
 
 // Scatter-combine of complex products: C blocks (interleaved complex) from the
-// quadrants of the doubled real C_q (one CTA per job).
-cudaError_t launch_cscatter(const CScatterJob *jobs, int64_t njobs, const double *wc, double *c,
-                            cudaStream_t stream);
+// quadrants of the doubled real C_q (one CTA per chunk of a job).
+cudaError_t launch_cscatter(const CScatterJob *jobs, const CScatterChunk *chunks, int64_t nchunks, const double *wc,
+                            double *c, cudaStream_t stream);
 
 // N(0, 1) numbers: Philox4x32-10 words turned by Box-Muller (see ytn_fill_normal).
 cudaError_t launch_fill_normal(uint64_t seed, int64_t n, double *out, cudaStream_t stream);

@@ -1114,6 +1114,7 @@ ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int n
   finalize_out(C, outb, off_of_id);
   // Scatter C: block (I, J) = C_q[row_off(I) + i, col_off(J) + j], row-major per leg.
   p->cs_jobs.clear();
+  p->cs_chunks.clear();
   for (size_t id = 0; id < srcs.size() && ca * cb > 1; id++) {
     // complex product: combine the quadrants of the doubled C_q
     const Src &sr = srcs[id];
@@ -1129,18 +1130,17 @@ ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int n
     J.q01 = cb == 2 ? g.N : -1;
     J.q10 = ca == 2 ? g.M * h.N : -1;
     J.q11 = (ca == 2 && cb == 2) ? g.M * h.N + g.N : -1;
-    J.nd = (int32_t)cd.size();
-    int64_t acc = 1;
-    for (int i = (int)freeA.size() - 1; i >= 0; i--) { J.sstr[i] = acc * h.N; acc *= cd[i]; }
-    acc = 1;
-    for (int i = (int)cd.size() - 1; i >= (int)freeA.size(); i--) { J.sstr[i] = acc; acc *= cd[i]; }
-    int64_t n = 1;
-    for (size_t i = 0; i < cd.size(); i++) {
-      J.ext[i] = (int32_t)cd[i];
-      n *= cd[i];
-    }
+    // A's free legs are the rows of the block in C_q, B's the columns: two dims
+    const int64_t n = sr.nI * sr.nJ;
     if (n > INT32_MAX) { err = "output block too large"; return YTN_E_UNSUPPORTED; }
+    J.ld = h.N;
     J.n = (int32_t)n;
+    J.nj = (int32_t)sr.nJ;
+    uint8_t shf = 0;
+    division_magic(sr.nJ, J.mag, shf);
+    J.shf = shf;
+    for (int64_t e = 0; e < n; e += kCScatterElems)
+      p->cs_chunks.push_back({(int32_t)p->cs_jobs.size(), (int32_t)e});
     p->cs_jobs.push_back(J);
     p->moved += n;
   }

@@ -234,15 +234,22 @@ static_assert(sizeof(SplitRecord) == 64, "SplitRecord layout");
 
 // Scatter of a complex product: one C block from the quadrants of the doubled
 // C_q (P = [[re.re, re.im], [im.re, im.im]] in rows x columns): element e of the
-// block (row-major over its nd dims) reads P at src + sum idx_i sstr_i plus the
+// block (nj columns, row-major) reads P at src + (e / nj) ld + e % nj plus the
 // quadrant offsets q01, q10, q11 (-1: quadrant absent, a real operand), and
-// writes re = P00 - P11, im = P01 + P10 at complex element dst + e.
+// writes re = P00 - P11, im = P01 + P10 at complex element dst + e. mag / shf divide
+// by nj (as in CopyJob). A CTA takes kCScatterElems elements of one job.
 struct CScatterJob {
   int64_t src, dst;
   int64_t q01, q10, q11;
-  int32_t nd, n;
-  int32_t ext[kMaxCopyDims];
-  int64_t sstr[kMaxCopyDims];
+  int64_t ld;
+  int32_t n, nj;
+  uint32_t mag;
+  int32_t shf;
+};
+static_assert(sizeof(CScatterJob) == 64, "CScatterJob layout");
+constexpr int kCScatterElems = 1024;
+struct CScatterChunk {
+  int32_t job, e0;
 };
 
 // ----------------------------------------------------------------------------
@@ -392,6 +399,7 @@ struct ytn_plan_s {
   // trace
   std::vector<ytn::TraceOut> tr_out;
   std::vector<ytn::CScatterJob> cs_jobs;   // complex tensordot: the scatter-combine
+  std::vector<ytn::CScatterChunk> cs_chunks;
   std::vector<ytn::TraceContrib> tr_contrib;
   std::vector<ytn::TraceChunk> tr_chunks;
   std::vector<ytn::VdotPiece> vd_pieces;
@@ -406,6 +414,7 @@ struct ytn_plan_s {
   const ytn::GemmTile *d_tiles = nullptr;
   const ytn::TraceOut *d_tr_out = nullptr;
   const ytn::CScatterJob *d_cs_jobs = nullptr;
+  const ytn::CScatterChunk *d_cs_chunks = nullptr;
   const ytn::TraceContrib *d_tr_contrib = nullptr;
   const ytn::TraceChunk *d_tr_chunks = nullptr;
   const ytn::VdotPiece *d_vd_pieces = nullptr;
