@@ -62,6 +62,11 @@ static ytn_status upload(ytn_plan_t *p) {
   put_table(buf, p->sectors_dev, o_sec);
   put_table(buf, p->tiles, o_tiles);
   put_table(buf, p->tr_out, o_tro);
+  size_t o_os, o_or, o_oc, o_ob;
+  put_table(buf, p->out_sec, o_os);
+  put_table(buf, p->out_rows, o_or);
+  put_table(buf, p->out_cols, o_oc);
+  put_table(buf, p->out_base, o_ob);
   size_t o_csj;
   put_table(buf, p->cs_jobs, o_csj);
   size_t o_csk;
@@ -98,6 +103,10 @@ static ytn_status upload(ytn_plan_t *p) {
   p->d_items = reinterpret_cast<const CopyItem *>(d + o_items);
   p->d_sectors = reinterpret_cast<const SectorDev *>(d + o_sec);
   p->d_tiles = reinterpret_cast<const GemmTile *>(d + o_tiles);
+  p->d_out_sec = reinterpret_cast<const SectorOut *>(d + o_os);
+  p->d_out_rows = reinterpret_cast<const OutRow *>(d + o_or);
+  p->d_out_cols = reinterpret_cast<const OutCol *>(d + o_oc);
+  p->d_out_base = reinterpret_cast<const int64_t *>(d + o_ob);
   p->d_tr_out = reinterpret_cast<const TraceOut *>(d + o_tro);
   p->d_cs_jobs = reinterpret_cast<const CScatterJob *>(d + o_csj);
   p->d_cs_chunks = reinterpret_cast<const CScatterChunk *>(d + o_csk);
@@ -726,16 +735,22 @@ ytn_status ytn_workspace_size(const ytn_plan_t *p, ytn_precision prec, double rt
   return fail(YTN_E_INVALID, "unknown precision");
 }
 
-// One contraction on the chosen path; arguments already checked and mapped.
+// One contraction on the chosen path; arguments already checked and mapped. direct:
+// the GEMM may write C's blocks itself (C in device memory); complex products and
+// results in host memory go through the dense C_q and a scatter, whose writes run
+// along the blocks.
 static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b, double *c, bool split, int slices,
-                                 double rtol, void *workspace, cudaStream_t st, bool fused_variant = false,
-                                 bool narrow_tails = false, bool pipelined = false) {
+                                 double rtol, void *workspace, cudaStream_t st, bool direct,
+                                 bool fused_variant = false, bool narrow_tails = false, bool pipelined = false) {
   WsLayout w;
   workspace_layout(p, split, w);
   char *ws = static_cast<char *>(workspace);
   double *wa = reinterpret_cast<double *>(ws + w.wa), *wb = reinterpret_cast<double *>(ws + w.wb),
          *wc = reinterpret_cast<double *>(ws + w.wc);
   cudaError_t e;
+  direct = direct && p->ca * p->cb == 1 && !split;
+  const OutView out = direct ? OutView{p->d_out_sec, p->d_out_rows, p->d_out_cols, p->d_out_base, c}
+                             : OutView{nullptr, nullptr, nullptr, nullptr, wc};
   // the fused split builds its slices straight from the blocks and gathers FP64
   // sector matrices only for the sectors its accuracy check recomputes
   const bool fused = split && p->sp_fused && fused_variant;
@@ -757,7 +772,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
   }
   if (!split) {
     PhaseTimer t(p->ctx, YTN_PHASE_GEMM, st);
-    e = launch_gemm_fp64(p->d_sectors, p->d_tiles, (int64_t)p->tiles.size(), wa, wb, wc, st);
+    e = launch_gemm_fp64(p->d_sectors, p->d_tiles, (int64_t)p->tiles.size(), wa, wb, out, st);
     if (e != cudaSuccess) return cuda_fail(e, "grouped FP64 GEMM");
   } else {
     int32_t *ea = reinterpret_cast<int32_t *>(ws + w.ea), *eb = reinterpret_cast<int32_t *>(ws + w.eb);
@@ -853,11 +868,11 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
                                   p->d_sp_sectors, p->d_sectors, flagged, item_end_a, item_end_b, rec, a, b, wa, wb,
                                   p->zero_a, p->zero_b, p->ctx->num_sms, st);
       if (e == cudaSuccess && !p->sp_sectors.empty())
-        e = launch_gemm_fp64_redo(p->d_sectors, flagged, tile_end, rec, wa, wb, wc, p->ctx->num_sms, st);
+        e = launch_gemm_fp64_redo(p->d_sectors, flagged, tile_end, rec, wa, wb, out, p->ctx->num_sms, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "accuracy check of the split products");
   }
-  {
+  if (!direct) {
     PhaseTimer t(p->ctx, YTN_PHASE_SCATTER, st);
     if (p->ca * p->cb > 1)
       e = launch_cscatter(p->d_cs_jobs, p->d_cs_chunks, (int64_t)p->cs_chunks.size(), wc, c, st);
@@ -955,6 +970,7 @@ ytn_status ytn_tensordot(ytn_plan_t *p, const double *a, const double *b, double
       if (hc) c = sc;
     }
   }
+  const bool direct = !hc || staged;   // C (or its staging copy) lies in device memory
   auto unstage = [&]() -> ytn_status {
     if (!staged || !hc || !p->out.size) return YTN_OK;
     const size_t wc = (size_t)p->out.size * (p->out.dtype == YTN_COMPLEX128 ? 16 : 8);
@@ -1012,16 +1028,16 @@ ytn_status ytn_tensordot(ytn_plan_t *p, const double *a, const double *b, double
     const bool with64 = need_choice, withfused = p->sp_fused && !((ha || hb) && !staged), withmix = has_mix;
     const bool withpipe = withfused && p->sp_pipe_tile_end.size() >= 2;
     std::vector<std::function<ytn_status()>> runs;
-    if (with64) runs.push_back([&]() { return exec_tensordot(p, a, b, c, false, 0, rtol, workspace, st); });
-    runs.push_back([&]() { return exec_tensordot(p, a, b, c, true, slices, rtol, workspace, st, false, false); });
+    if (with64) runs.push_back([&]() { return exec_tensordot(p, a, b, c, false, 0, rtol, workspace, st, direct); });
+    runs.push_back([&]() { return exec_tensordot(p, a, b, c, true, slices, rtol, workspace, st, direct, false, false); });
     if (withfused)
-      runs.push_back([&]() { return exec_tensordot(p, a, b, c, true, slices, rtol, workspace, st, true, false); });
+      runs.push_back([&]() { return exec_tensordot(p, a, b, c, true, slices, rtol, workspace, st, direct, true, false); });
     if (withpipe)
       runs.push_back(
-          [&]() { return exec_tensordot(p, a, b, c, true, slices, rtol, workspace, st, true, false, true); });
+          [&]() { return exec_tensordot(p, a, b, c, true, slices, rtol, workspace, st, direct, true, false, true); });
     if (withmix)
       runs.push_back(
-          [&]() { return exec_tensordot(p, a, b, c, true, slices, rtol, workspace, st, withfused, true); });
+          [&]() { return exec_tensordot(p, a, b, c, true, slices, rtol, workspace, st, direct, withfused, true); });
     // one round of the candidates; short contractions (a round under 20 ms) get two
     // more and keep each candidate's fastest, so that launch jitter does not decide
     std::vector<float> ms;
@@ -1081,7 +1097,8 @@ ytn_status ytn_tensordot(ytn_plan_t *p, const double *a, const double *b, double
   const bool use_pipe = use_fused && variant == 2 && !capturing;
   const bool use_mix = split && has_mix && tiles == 1 && !use_pipe;
   ytn_status r =
-      exec_tensordot(p, a, b, c, split, split ? slices : 0, rtol, workspace, st, use_fused, use_mix, use_pipe);
+      exec_tensordot(p, a, b, c, split, split ? slices : 0, rtol, workspace, st, direct, use_fused, use_mix,
+                     use_pipe);
   if (r != YTN_OK) return r;
   if ((r = unstage()) != YTN_OK) return r;
   fill_res(split, use_pipe ? 2 : use_fused ? 1 : 0);

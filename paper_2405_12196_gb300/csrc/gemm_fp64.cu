@@ -3,17 +3,24 @@
 // tensor cores (DMMA, mma.sync m8n8k4 f64).
 //
 // One launch covers every sector: the grid is the host-built tile list
-// (sector, m-tile, n-tile), largest K first so that long tiles start early.
+// (sector, m-tile, n-tile), largest tiles first so that long ones start early.
 // Each CTA computes one tile of C_q over the full K (no split-K), so every
 // output element has one fixed summation order: results do not depend on the
-// schedule or on what else runs on the GPU. The tile edge (64, or 32 for small
-// and thin sectors) is chosen per sector by the planner from the sector's M and
-// N, so that many small sectors do not pay for 64x64 tiles.
+// schedule, the tile edge or on what else runs on the GPU. The tile edge (64, 32 or
+// 16) is chosen per sector by the planner so that the work spreads over the SMs.
 //
-// On GB300 the FP64 rate (DMMA and DFMA alike, about 1 TFLOP/s for the whole
-// GPU) is low enough that this kernel is bound by the FP64 pipe even at 64x64
-// tiles; operands are staged through padded shared memory with a register
-// prefetch of the next K step.
+// On GB300 the FP64 rate (DMMA and DFMA alike, about 1 TFLOP/s for the whole GPU: two
+// multiply-adds per clock and SM) is low enough that this kernel is bound by the FP64
+// pipe at every tile edge; operands are staged through padded shared memory with a
+// register prefetch of the next K step. So no padding is multiplied: DMMA blocks
+// outside the sector are skipped, K advances in steps of 4 to its end, and sectors
+// with K <= 2 (double layers contracted over a physical leg: one element per charge)
+// take plain multiply-adds, one per K, instead of a DMMA step of 4. The Z2 D = 8
+// double layer (2 sectors of 2048 x 2048 x 1) took 260 us with K padded to 16 and
+// takes 50 us.
+//
+// The epilogue writes C's blocks directly through the planner's row, column and block
+// tables (OutView), or the dense C_q of the workspace when a scatter follows.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -72,11 +79,53 @@ __device__ __forceinline__ void store_tile(double (*s)[64 + PAD], const double (
   }
 }
 
-// One T x T tile of C_q (T = 64 or 32): four warps of (T/2) x (T/2), each a grid of
-// (T/16) x (T/16) DMMA 8x8 blocks.
+// A warp's accumulators (8 x 8 DMMA blocks; the thread's elements are rows m + 8 i,
+// columns n + 8 j and the next one) into C.
+template <int NB>
+__device__ __forceinline__ void store_tile_out(const SectorDev &s, int sector, const OutView &out,
+                                               const double (&acc)[NB][NB][2], int m, int n) {
+  if (!out.sec) {   // the dense C_q
+    double *C = out.c + s.c_off;
+#pragma unroll
+    for (int i = 0; i < NB; i++) {
+      if (m + 8 * i >= s.M) continue;
+      double *row = C + (int64_t)(m + 8 * i) * s.N;
+#pragma unroll
+      for (int j = 0; j < NB; j++)
+#pragma unroll
+        for (int h = 0; h < 2; h++)
+          if (n + 8 * j + h < s.N) row[n + 8 * j + h] = acc[i][j][h];
+    }
+    return;
+  }
+  const SectorOut so = out.sec[sector];
+  OutCol col[NB][2];
+#pragma unroll
+  for (int j = 0; j < NB; j++)
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+      if (n + 8 * j + h < s.N) col[j][h] = out.cols[so.cols + n + 8 * j + h];
+#pragma unroll
+  for (int i = 0; i < NB; i++) {
+    if (m + 8 * i >= s.M) continue;
+    const OutRow row = out.rows[so.rows + m + 8 * i];
+    const int64_t *base = out.base + so.base + (int64_t)row.blk * so.ncb;
+#pragma unroll
+    for (int j = 0; j < NB; j++)
+#pragma unroll
+      for (int h = 0; h < 2; h++)
+        if (n + 8 * j + h < s.N) {
+          const int64_t b = __ldg(base + col[j][h].blk);
+          if (b >= 0) out.c[b + (int64_t)row.idx * col[j][h].len + col[j][h].idx] = acc[i][j][h];
+        }
+  }
+}
+
+// One T x T tile of C_q (T = 64, 32 or 16): four warps of (T/2) x (T/2), each a grid
+// of (T/16) x (T/16) DMMA 8x8 blocks.
 template <int T>
 __device__ __forceinline__ void gemm_tile(const SectorDev &s, const GemmTile &tl, const double *__restrict__ wa,
-                                          const double *__restrict__ wb, double *__restrict__ wc,
+                                          const double *__restrict__ wb, const OutView &out,
                                           double (*As)[BK][64 + PAD], double (*Bs)[BK][64 + PAD]) {
   constexpr int NB = T / 16;
   const int M = s.M, N = s.N, K = s.K;
@@ -95,6 +144,8 @@ __device__ __forceinline__ void gemm_tile(const SectorDev &s, const GemmTile &tl
 #pragma unroll
     for (int j = 0; j < NB; j++) acc[i][j][0] = acc[i][j][1] = 0.0;
 
+  // DMMA blocks of this warp that meet the sector (the same for the whole warp)
+  const int nbm = (M - m0 - wm + 7) >> 3, nbn = (N - n0 - wn + 7) >> 3;
   double ra[T / 8], rb[T / 8];
   const int nk = (K + BK - 1) / BK;
   if (nk > 0) {
@@ -111,8 +162,10 @@ __device__ __forceinline__ void gemm_tile(const SectorDev &s, const GemmTile &tl
       load_tile<T>(ra, A, lda, akm, M, m0, (kt + 1) * BK, K);
       load_tile<T>(rb, B, ldb, bkm, N, n0, (kt + 1) * BK, K);
     }
+    const int kend = min(BK, K - kt * BK);   // steps of 4 beyond K hold zeros only
 #pragma unroll
     for (int kk = 0; kk < BK; kk += 4) {
+      if (kk >= kend) break;
       double af[NB], bf[NB];
 #pragma unroll
       for (int i = 0; i < NB; i++) af[i] = As[cur][kk + (lane & 3)][wm + i * 8 + (lane >> 2)];
@@ -121,7 +174,8 @@ __device__ __forceinline__ void gemm_tile(const SectorDev &s, const GemmTile &tl
 #pragma unroll
       for (int i = 0; i < NB; i++)
 #pragma unroll
-        for (int j = 0; j < NB; j++) dmma(acc[i][j], af[i], bf[j]);
+        for (int j = 0; j < NB; j++)
+          if (i < nbm && j < nbn) dmma(acc[i][j], af[i], bf[j]);
     }
     if (more) {
       store_tile<T>(As[cur ^ 1], ra, akm);
@@ -129,31 +183,64 @@ __device__ __forceinline__ void gemm_tile(const SectorDev &s, const GemmTile &tl
     }
     __syncthreads();
   }
-  double *C = wc + s.c_off;
+  store_tile_out<NB>(s, tl.sector, out, acc, m0 + wm + (lane >> 2), n0 + wn + 2 * (lane & 3));
+}
+
+// Sectors with K <= 2: one 64 x 64 tile by 128 threads, thread t the rows of its half
+// (t / 64, every second one) at column t % 64, so that the stores of a warp run along
+// the columns. The products are summed in the order of k, as the DMMA steps do.
+constexpr int kOuterK = 2;
+
+__device__ __forceinline__ void outer_tile(const SectorDev &s, const GemmTile &tl, const double *__restrict__ wa,
+                                           const double *__restrict__ wb, const OutView &out, double (*As)[64],
+                                           OutRow *rows) {
+  const int M = s.M, N = s.N, K = s.K, t = threadIdx.x;
+  const int m0 = tl.mt * 64, n = tl.nt * 64 + (t & 63);
+  const int nr = min(64, M - m0);
+  const bool direct = out.sec != nullptr;
+  const SectorOut so = direct ? out.sec[tl.sector] : SectorOut{};
+  for (int e = t; e < nr * K; e += kThreads) {
+    const int r = e / K, k = e - r * K;
+    As[k][r] = wa[s.a_off + (s.a_kmajor ? (int64_t)(m0 + r) * K + k : (int64_t)k * M + m0 + r)];
+  }
+  if (t < nr) rows[t] = direct ? out.rows[so.rows + m0 + t] : OutRow{0, m0 + t};
+  __syncthreads();
+  if (n >= N) return;
+  double b[kOuterK];
 #pragma unroll
-  for (int i = 0; i < NB; i++) {
-    const int m = m0 + wm + i * 8 + (lane >> 2);
-    if (m >= M) continue;
-#pragma unroll
-    for (int j = 0; j < NB; j++) {
-      const int n = n0 + wn + j * 8 + 2 * (lane & 3);
-      if (n < N) C[(int64_t)m * N + n] = acc[i][j][0];
-      if (n + 1 < N) C[(int64_t)m * N + n + 1] = acc[i][j][1];
+  for (int k = 0; k < kOuterK; k++)
+    b[k] = k < K ? __ldg(wb + s.b_off + (s.b_kmajor ? (int64_t)n * K + k : (int64_t)k * N + n)) : 0.0;
+  const OutCol col = direct ? out.cols[so.cols + n] : OutCol{0, n, N, 0};
+  int blk = -1;
+  int64_t base = s.c_off;
+  if (!direct) blk = 0;
+#pragma unroll 4
+  for (int r = t >> 6; r < nr; r += 2) {
+    const OutRow row = rows[r];
+    if (row.blk != blk) {
+      blk = row.blk;
+      base = __ldg(out.base + so.base + (int64_t)blk * so.ncb + col.blk);
     }
+    double v = As[0][r] * b[0];
+    if (K > 1) v = fma(As[1][r], b[1], v);
+    if (base >= 0) out.c[base + (int64_t)row.idx * col.len + col.idx] = v;
   }
 }
 
 __global__ void __launch_bounds__(kThreads) gemm_fp64_kernel(const SectorDev *__restrict__ sectors,
                                                              const GemmTile *__restrict__ tiles,
                                                              const double *__restrict__ wa,
-                                                             const double *__restrict__ wb,
-                                                             double *__restrict__ wc) {
+                                                             const double *__restrict__ wb, OutView out) {
   __shared__ double As[2][BK][64 + PAD];
   __shared__ double Bs[2][BK][64 + PAD];
   const GemmTile tl = tiles[blockIdx.x];
   const SectorDev s = sectors[tl.sector];
-  if (tl.size == 32) gemm_tile<32>(s, tl, wa, wb, wc, As, Bs);
-  else gemm_tile<64>(s, tl, wa, wb, wc, As, Bs);
+  if (tl.size == 16) gemm_tile<16>(s, tl, wa, wb, out, As, Bs);
+  else if (tl.size == 32) gemm_tile<32>(s, tl, wa, wb, out, As, Bs);
+  else if (s.K <= kOuterK)
+    outer_tile(s, tl, wa, wb, out, reinterpret_cast<double(*)[64]>(&As[0][0][0]),
+               reinterpret_cast<OutRow *>(&Bs[0][0][0]));
+  else gemm_tile<64>(s, tl, wa, wb, out, As, Bs);
 }
 
 // FP64 recomputation of the sectors that the split path's accuracy check
@@ -165,8 +252,7 @@ __global__ void __launch_bounds__(kThreads) gemm_fp64_redo_kernel(const SectorDe
                                                                   const int32_t *__restrict__ tile_end,
                                                                   const SplitRecord *__restrict__ rec,
                                                                   const double *__restrict__ wa,
-                                                                  const double *__restrict__ wb,
-                                                                  double *__restrict__ wc) {
+                                                                  const double *__restrict__ wb, OutView out) {
   __shared__ double As[2][BK][64 + PAD];
   __shared__ double Bs[2][BK][64 + PAD];
   const int nflag = rec->nfallback;
@@ -183,7 +269,7 @@ __global__ void __launch_bounds__(kThreads) gemm_fp64_redo_kernel(const SectorDe
     const SectorDev s = sectors[flagged[lo]];
     const int nt = (s.N + 63) / 64;
     const GemmTile tl{flagged[lo], local / nt, local % nt, 64};
-    gemm_tile<64>(s, tl, wa, wb, wc, As, Bs);
+    gemm_tile<64>(s, tl, wa, wb, out, As, Bs);
     __syncthreads();
   }
 }
@@ -191,18 +277,18 @@ __global__ void __launch_bounds__(kThreads) gemm_fp64_redo_kernel(const SectorDe
 }  // namespace
 
 cudaError_t launch_gemm_fp64_redo(const SectorDev *sectors, const int32_t *flagged, const int32_t *tile_end,
-                                  const SplitRecord *rec, const double *wa, const double *wb, double *wc,
+                                  const SplitRecord *rec, const double *wa, const double *wb, const OutView &out,
                                   int num_sms, cudaStream_t stream) {
   gemm_fp64_redo_kernel<<<(unsigned)std::max(1, num_sms) * 4, kThreads, 0, stream>>>(sectors, flagged, tile_end, rec,
-                                                                                    wa, wb, wc);
+                                                                                    wa, wb, out);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gemm_fp64(const SectorDev *sectors, const GemmTile *tiles, int64_t ntiles,
-                             const double *wa, const double *wb, double *wc, cudaStream_t stream) {
+                             const double *wa, const double *wb, const OutView &out, cudaStream_t stream) {
   if (ntiles <= 0) return cudaSuccess;
   if (ntiles > INT32_MAX) return cudaErrorInvalidValue;
-  gemm_fp64_kernel<<<(unsigned)ntiles, kThreads, 0, stream>>>(sectors, tiles, wa, wb, wc);
+  gemm_fp64_kernel<<<(unsigned)ntiles, kThreads, 0, stream>>>(sectors, tiles, wa, wb, out);
   return cudaGetLastError();
 }
 

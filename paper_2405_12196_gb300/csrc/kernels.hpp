@@ -22,9 +22,10 @@ cudaError_t launch_trace(const TraceChunk *chunks, int64_t nchunks, const TraceO
 cudaError_t launch_vdot(const VdotChunk *chunks, int64_t nchunks, const VdotPiece *pieces, const double *a,
                         const double *b, double *partials, double *out, bool complex_data, cudaStream_t stream);
 
-// Grouped FP64 GEMM (DMMA) over 64x64 tiles: C_q = A_q B_q.
+// Grouped FP64 GEMM (DMMA) over the tile list: C_q = A_q B_q, into C's blocks or the
+// dense C_q (see OutView).
 cudaError_t launch_gemm_fp64(const SectorDev *sectors, const GemmTile *tiles, int64_t ntiles,
-                             const double *wa, const double *wb, double *wc, cudaStream_t stream);
+                             const double *wa, const double *wb, const OutView &out, cudaStream_t stream);
 
 // Split-precision path: row exponents and BF16 slices of every sector operand.
 // Staged path (from the FP64 sector matrices wa, wb): row exponents (ea, eb;
@@ -90,7 +91,7 @@ cudaError_t launch_gather_flagged(const CopyJob *jobs, const CopyItem *items_a, 
 // FP64 recomputation of the flagged sectors (persistent, 64 x 64 DMMA tiles):
 // the sector list and tile counts come from the accuracy check on the device.
 cudaError_t launch_gemm_fp64_redo(const SectorDev *sectors, const int32_t *flagged, const int32_t *tile_end,
-                                  const SplitRecord *rec, const double *wa, const double *wb, double *wc,
+                                  const SplitRecord *rec, const double *wa, const double *wb, const OutView &out,
                                   int num_sms, cudaStream_t stream);
 
 }  // namespace ytn

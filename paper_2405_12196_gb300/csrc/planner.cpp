@@ -1068,7 +1068,12 @@ ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int n
 
   // Output blocks: (I, J) exists when some x has both A(I, x) and B(x, J).
   std::vector<OutBlock> outb;
-  struct Src { int64_t sector; int64_t roff, coff; int64_t nI, nJ; int64_t a_blk, b_blk; };
+  struct Src { int64_t sector; int64_t roff, coff; int64_t nI, nJ; int64_t a_blk, b_blk; int64_t base; };
+  const bool direct = ca * cb == 1;   // the GEMMs write C's blocks themselves
+  p->out_sec.clear();
+  p->out_rows.clear();
+  p->out_cols.clear();
+  p->out_base.clear();
   std::vector<Src> srcs;
   for (size_t si = 0; si < geo.size(); si++) {
     const SG &g = geo[si];
@@ -1091,9 +1096,28 @@ ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int n
         v[xi / 64] |= 1ull << (xi % 64);
       }
     }
+    int64_t base = 0;   // this sector's table of block offsets, filled once C is laid out
+    if (direct) {
+      base = (int64_t)p->out_base.size();
+      p->out_sec.push_back({(int64_t)p->out_rows.size(), (int64_t)p->out_cols.size(), base, (int32_t)sb.cols.size(), 0});
+      p->out_base.resize(p->out_base.size() + sb.rows.size() * sb.cols.size(), -1);
+      int32_t blk = 0;
+      for (auto &r : sb.rows) {
+        for (int64_t i = 0; i < r.second.first; i++) p->out_rows.push_back({blk, (int32_t)i});
+        blk++;
+      }
+      blk = 0;
+      for (auto &c : sb.cols) {
+        for (int64_t j = 0; j < c.second.first; j++)
+          p->out_cols.push_back({blk, (int32_t)j, (int32_t)c.second.first, 0});
+        blk++;
+      }
+    }
+    int64_t at = -1;   // (row block, column block) in the sector's table
     for (auto &r : sb.rows) {
       const auto &rv = rowx[r.first];
       for (auto &c : sb.cols) {
+        at++;
         const auto &cv = colx[c.first];
         bool hit = false;
         for (int w = 0; w < nw && !hit; w++) hit = (rv[w] & cv[w]) != 0;
@@ -1106,13 +1130,15 @@ ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int n
         ob.id = (int64_t)srcs.size();
         outb.push_back(ob);
         srcs.push_back({(int64_t)si, g.row_off.at(r.first), g.col_off.at(c.first), r.second.first,
-                        c.second.first, r.second.second, c.second.second});
+                        c.second.first, r.second.second, c.second.second, base + at});
       }
     }
   }
   std::vector<int64_t> off_of_id;
   finalize_out(C, outb, off_of_id);
-  // Scatter C: block (I, J) = C_q[row_off(I) + i, col_off(J) + j], row-major per leg.
+  if (direct)
+    for (size_t id = 0; id < srcs.size(); id++) p->out_base[srcs[id].base] = off_of_id[id];
+  // Scatter C (into host memory; else the GEMMs write it): block (I, J) = C_q[row_off(I) + i, col_off(J) + j], row-major per leg.
   p->cs_jobs.clear();
   p->cs_chunks.clear();
   for (size_t id = 0; id < srcs.size() && ca * cb > 1; id++) {
@@ -1172,20 +1198,27 @@ ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int n
   make_items(p, j2, j3);
   p->items_c_end = (int64_t)p->items.size();
 
-  // Grouped-GEMM tiles, largest K first. The tile edge is chosen per sector from
-  // its size: 32 when 32 x 32 tiles cover the sector with at most 60% of the
-  // padded area of 64 x 64 tiles (small or thin M, N), else 64.
+  // Grouped-GEMM tiles, largest first. The kernel is bound by the FP64 pipe of each
+  // SM at every tile edge (an SM does two FP64 multiply-adds per clock; a 16 x 16 tile
+  // loads 0.55 TB/s over the whole GPU at that rate), and skips the 8 x 8 blocks
+  // outside the sector, so the edge only decides how evenly the work spreads: the
+  // largest of 64, 32, 16 whose tile is at most a quarter of an SM's share of the
+  // plan's work (17 ragged sectors up to 251 x 188 x 188: 64 x 64 tiles kept 64 of 152
+  // SMs busy, 229 us; 16 x 16 62 us).
   p->tiles.clear();
+  double work = 0.0;
+  for (const HostSector &h : p->sectors) work += (double)((h.M + 7) / 8 * 8) * ((h.N + 7) / 8 * 8) * h.K;
+  const double share = work / std::max(1, p->ctx ? p->ctx->num_sms : 0);
   for (size_t si = 0; si < geo.size(); si++) {
     const int64_t M = p->sectors[si].M, N = p->sectors[si].N;
-    const int64_t a64 = ((M + 63) / 64) * ((N + 63) / 64) * 4096, a32 = ((M + 31) / 32) * ((N + 31) / 32) * 1024;
-    const int T = 10 * a32 <= 6 * a64 ? 32 : 64;
+    int T = 64;
+    while (T > 16 && 4.0 * T * T * p->sectors[si].K > share) T /= 2;
     const int64_t mt = (M + T - 1) / T, nt = (N + T - 1) / T;
     for (int64_t i = 0; i < mt; i++)
       for (int64_t j = 0; j < nt; j++) p->tiles.push_back({(int32_t)si, (int32_t)i, (int32_t)j, T});
   }
   std::stable_sort(p->tiles.begin(), p->tiles.end(), [&](const GemmTile &x, const GemmTile &y) {
-    return geo[x.sector].K > geo[y.sector].K;
+    return (int64_t)x.size * x.size * geo[x.sector].K > (int64_t)y.size * y.size * geo[y.sector].K;
   });
   plan_split_tables(p, seg_src);
   p->kind = Kind::Tensordot;

@@ -79,11 +79,38 @@ struct SectorDev {
 };
 static_assert(sizeof(SectorDev) == 48, "SectorDev layout");
 
+// Where the elements of a sector's C_q lie in C's blocks, so that the GEMMs write C
+// itself: row m belongs to row block `blk` (a charge tuple of A's free legs) at row
+// idx inside it, column n to column block `blk` of `len` columns at column idx, and
+// block (I, J) starts at element base[I * ncb + J] of C (-1: no such block) with
+// row-major elements, so C_q[m][n] is at base + idx_m * len_n + idx_n. The tables of
+// all sectors lie back to back; a SectorOut holds a sector's offsets into them.
+struct OutRow {
+  int32_t blk, idx;
+};
+struct OutCol {
+  int32_t blk, idx, len, pad;
+};
+struct SectorOut {
+  int64_t rows, cols, base;
+  int32_t ncb, pad;
+};
+// The tables on the device and the destination: C's data (tables set), or with null
+// tables the dense sector matrices of the workspace (row-major at SectorDev::c_off;
+// complex products and results in host memory, scattered by the copy kernels).
+struct OutView {
+  const SectorOut *sec;
+  const OutRow *rows;
+  const OutCol *cols;
+  const int64_t *base;
+  double *c;
+};
+
 // One output tile of the grouped FP64 GEMM.
 struct GemmTile {
   int32_t sector;
   int32_t mt, nt;   // tile coordinates in units of `size`
-  int32_t size;     // tile edge: 64, or 32 for small sectors
+  int32_t size;     // tile edge: 64, 32 or 16
 };
 
 // Trace: one output block, fed by ncontrib contributing input blocks with nterms
@@ -405,6 +432,12 @@ struct ytn_plan_s {
   std::vector<ytn::VdotPiece> vd_pieces;
   std::vector<ytn::VdotChunk> vd_chunks;
 
+  // real tensordot: C's blocks as the GEMMs address them (empty for complex products)
+  std::vector<ytn::SectorOut> out_sec;
+  std::vector<ytn::OutRow> out_rows;
+  std::vector<ytn::OutCol> out_cols;
+  std::vector<int64_t> out_base;
+
   // device copies of the tables (one allocation)
   void *dev = nullptr;
   size_t dev_bytes = 0;
@@ -412,6 +445,10 @@ struct ytn_plan_s {
   const ytn::CopyItem *d_items = nullptr;
   const ytn::SectorDev *d_sectors = nullptr;
   const ytn::GemmTile *d_tiles = nullptr;
+  const ytn::SectorOut *d_out_sec = nullptr;
+  const ytn::OutRow *d_out_rows = nullptr;
+  const ytn::OutCol *d_out_cols = nullptr;
+  const int64_t *d_out_base = nullptr;
   const ytn::TraceOut *d_tr_out = nullptr;
   const ytn::CScatterJob *d_cs_jobs = nullptr;
   const ytn::CScatterChunk *d_cs_chunks = nullptr;
