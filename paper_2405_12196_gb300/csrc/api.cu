@@ -748,7 +748,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
   double *wa = reinterpret_cast<double *>(ws + w.wa), *wb = reinterpret_cast<double *>(ws + w.wb),
          *wc = reinterpret_cast<double *>(ws + w.wc);
   cudaError_t e;
-  direct = direct && p->ca * p->cb == 1 && !split;
+  direct = direct && p->ca * p->cb == 1;
   const OutView out = direct ? OutView{p->d_out_sec, p->d_out_rows, p->d_out_cols, p->d_out_base, c}
                              : OutView{nullptr, nullptr, nullptr, nullptr, wc};
   // the fused split builds its slices straight from the blocks and gathers FP64
@@ -806,7 +806,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
       if (e != cudaSuccess) return cuda_fail(e, "split into slices");
       {
         PhaseTimer t(p->ctx, YTN_PHASE_GEMM, hi);
-        e = launch_gemm_split(p->d_sp_sectors, p->d_sp_tiles, te[0], sa, sb, ea, eb, emax, normsq, wc, slices,
+        e = launch_gemm_split(p->d_sp_sectors, p->d_sp_tiles, te[0], sa, sb, ea, eb, emax, normsq, out, slices,
                               p->ctx->status_dev, sms, false, hi);
         // enqueued after group 0's GEMM, so that its CTAs are dispatched first
         if (e == cudaSuccess) e = cudaStreamWaitEvent(lo, ev(1), 0);
@@ -819,7 +819,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
           e = cudaStreamWaitEvent(hi, ev(g + 1), 0);
           if (e == cudaSuccess)
             e = launch_gemm_split(p->d_sp_sectors, p->d_sp_tiles + te[g - 1], te[g] - te[g - 1], sa, sb, ea, eb, emax,
-                                  normsq, wc, slices, p->ctx->status_dev, sms, false, hi);
+                                  normsq, out, slices, p->ctx->status_dev, sms, false, hi);
         }
       }
       if (e == cudaSuccess) e = cudaEventRecord(ev(ngroups + 1), hi);
@@ -849,7 +849,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
         const bool mix = narrow_tails && !p->sp_tiles_mix.empty();
         e = launch_gemm_split(p->d_sp_sectors, mix ? p->d_sp_tiles_mix : p->d_sp_tiles,
                               (int64_t)(mix ? p->sp_tiles_mix.size() : p->sp_tiles.size()), sa, sb, ea, eb, emax,
-                              normsq, wc, slices, p->ctx->status_dev, sms, mix, st);
+                              normsq, out, slices, p->ctx->status_dev, sms, mix, st);
       }
       if (e != cudaSuccess) return cuda_fail(e, "grouped split-precision GEMM");
     }
@@ -970,7 +970,15 @@ ytn_status ytn_tensordot(ytn_plan_t *p, const double *a, const double *b, double
       if (hc) c = sc;
     }
   }
-  const bool direct = !hc || staged;   // C (or its staging copy) lies in device memory
+  // the GEMM may write C's blocks: C (or its staging copy) lies in device memory, apart
+  // from the operands (the split path's FP64 recomputation reads them after the GEMM)
+  const size_t bytes_a = p->a_size * (p->ca == 2 ? 16 : 8), bytes_b = p->b_size * (p->cb == 2 ? 16 : 8);
+  const size_t bytes_c = (size_t)p->out.size * (p->out.dtype == YTN_COMPLEX128 ? 16 : 8);
+  auto apart = [&](const double *x, size_t n) {
+    const char *p0 = reinterpret_cast<const char *>(x), *c0 = reinterpret_cast<const char *>(c);
+    return p0 + n <= c0 || c0 + bytes_c <= p0;
+  };
+  const bool direct = (!hc || staged) && apart(a, bytes_a) && apart(b, bytes_b);
   auto unstage = [&]() -> ytn_status {
     if (!staged || !hc || !p->out.size) return YTN_OK;
     const size_t wc = (size_t)p->out.size * (p->out.dtype == YTN_COMPLEX128 ? 16 : 8);

@@ -57,14 +57,14 @@ cudaError_t launch_cscatter(const CScatterJob *jobs, const CScatterChunk *chunks
 // N(0, 1) numbers: Philox4x32-10 words turned by Box-Muller (see ytn_fill_normal).
 cudaError_t launch_fill_normal(uint64_t seed, int64_t n, double *out, cudaStream_t stream);
 
-// Split-precision grouped GEMM (tcgen05) over 128x128 tiles (and 128x64 tiles
-// when mixed_widths: the tile list holds them), FP64 output C_q;
-// the epilogue adds each sector's scaled ||C_q||^2 into normsq (emax: the
-// operands' largest exponents).
+// Split-precision grouped GEMM (tcgen05) over 256x128 tiles of CTA pairs (and 256x64
+// tiles when mixed_widths: the tile list holds them), FP64 output into C's blocks or
+// the dense C_q (see OutView); the epilogue adds each sector's scaled ||C_q||^2 into
+// normsq (emax: the operands' largest exponents).
 cudaError_t launch_gemm_split(const SplitSector *sectors, const SplitTile *tiles, int64_t ntiles, const uint8_t *sa,
                               const uint8_t *sb, const int32_t *ea, const int32_t *eb, const int32_t *emax,
-                              float *normsq, double *wc, int slices, int *status, int num_sms, bool mixed_widths,
-                              cudaStream_t stream);
+                              float *normsq, const OutView &out, int slices, int *status, int num_sms,
+                              bool mixed_widths, cudaStream_t stream);
 
 // Accuracy check of the split products (one CTA per sector, the last one
 // finalises): per-sector estimates from the exponents and normsq, the list of

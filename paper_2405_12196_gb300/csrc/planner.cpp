@@ -1229,8 +1229,8 @@ ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int n
 
 // Tables of the split-precision path: per sector, the slice blocks and exponents
 // of A (rows M) and B (rows N), the exponent / slicing work items and the
-// 128 x 128 output tiles (sectors by decreasing K; inside a sector, groups of 8
-// row tiles with the column tiles innermost, so that CTAs running at the same time
+// 256 x 128 output tiles (sectors by decreasing K; inside a sector, groups of 8
+// row tiles for each pair of column tiles, so that CTAs running at the same time
 // share operand slices in L2). When every block's dims fit kFusedDims per side,
 // also the fused path's items and segments (slices straight from the blocks).
 void plan_split_tables(ytn_plan_t *p, std::vector<SegSource> *src) {
@@ -1294,8 +1294,9 @@ void plan_split_tables(ytn_plan_t *p, std::vector<SegSource> *src) {
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(),
                    [&](int64_t x, int64_t y) { return p->sectors[x].K > p->sectors[y].K; });
-  // Tile lists: all 128 wide, and the same with the last column tile of a sector 64
-  // wide where the sector's N ends in its first half (N mod 128 in 1..64: half of the
+  // Tile lists: 256 columns x 128 rows of C_q per tile everywhere; and the same except
+  // for sectors whose N ends in the first half of a 128-wide tile (N mod 128 in 1..64),
+  // which take 256 rows x 128 columns with a last column tile 64 wide (half of the
   // padded products of that tile saved). The first split call on a plan times both
   // when they differ and keeps the faster.
   p->sp_tiles_mix.clear();
@@ -1305,15 +1306,41 @@ void plan_split_tables(ytn_plan_t *p, std::vector<SegSource> *src) {
     const int64_t tm = (h.M + kSplitBM - 1) / kSplitBM, tn = (h.N + kSplitBM - 1) / kSplitBM;
     const bool tail_narrow = h.N % kSplitBM != 0 && h.N % kSplitBM <= kSplitBM / 2;
     any_narrow = any_narrow || tail_narrow;
+    // tile (pt, qt) of width bn; swap: P is A, Q is B
+    auto tile = [&](int64_t pt, int64_t qt, int bn, bool swap) {
+      const SplitSector &sc = p->sp_sectors[q];
+      const SectorOut so = p->out_sec.empty() ? SectorOut{} : p->out_sec[q];
+      const int64_t p0 = 2 * kSplitBM * pt, q0 = bn * qt;
+      SplitTile t{};
+      t.sector = (int32_t)q;
+      t.pt = (int32_t)pt;
+      t.qt = (int32_t)qt;
+      t.bn = (int16_t)bn;
+      t.swap = swap ? 1 : 0;
+      t.ks = sc.ks;
+      t.np = (int32_t)((swap ? h.M : h.N) - p0);
+      t.nq = (int32_t)((swap ? h.N : h.M) - q0);
+      t.q_first = (int32_t)q0;
+      t.p_exp = (swap ? sc.ea_off : sc.eb_off) + p0;
+      t.q_exp = (swap ? sc.eb_off : sc.ea_off) + q0;
+      t.p_rec = (swap ? so.rows : so.cols) + p0;
+      t.q_rec = (swap ? so.cols : so.rows) + q0;
+      t.base = so.base;
+      t.c_off = h.c_off;
+      t.ncb = so.ncb;
+      t.ld = (int32_t)h.N;
+      return t;
+    };
     for (int64_t g0 = 0; g0 < tm; g0 += 8)
-      for (int64_t n = 0; n < tn; n++)
+      for (int64_t n = 0; n < (tn + 1) / 2; n++)
         for (int64_t m = g0; m < std::min<int64_t>(g0 + 8, tm); m++) {
-          p->sp_tiles.push_back({(int32_t)q, (int32_t)m, (int32_t)n, kSplitBM});
-          if (tail_narrow && n == tn - 1)
-            p->sp_tiles_mix.push_back({(int32_t)q, (int32_t)m, (int32_t)(2 * n), kSplitBM / 2});
-          else
-            p->sp_tiles_mix.push_back({(int32_t)q, (int32_t)m, (int32_t)n, kSplitBM});
+          p->sp_tiles.push_back(tile(n, m, kSplitBM, false));
+          if (!tail_narrow) p->sp_tiles_mix.push_back(p->sp_tiles.back());
         }
+    for (int64_t g0 = 0; tail_narrow && g0 < tn; g0 += 8)
+      for (int64_t m = 0; m < (tm + 1) / 2; m++)
+        for (int64_t n = g0; n < std::min<int64_t>(g0 + 8, tn); n++)
+          p->sp_tiles_mix.push_back(n == tn - 1 ? tile(m, 2 * n, kSplitBM / 2, true) : tile(m, n, kSplitBM, true));
   }
   if (!any_narrow) p->sp_tiles_mix.clear();
 
@@ -1434,17 +1461,17 @@ void plan_split_tables(ytn_plan_t *p, std::vector<SegSource> *src) {
   p->sp_fused = true;
 
   // Pipeline groups: runs of sectors in the GEMM's order of about an eighth of the
-  // useful FLOPs each, every group holding at least two waves of 128-wide tiles
-  // (one CTA per SM), so that each group's GEMM launch fills the GPU; the last run
+  // useful FLOPs each, every group holding at least two waves of 256 x 128 tiles
+  // (one pair of CTAs per two SMs), so that each group's GEMM launch fills the GPU; the last run
   // joins its predecessor when it is shorter. Fewer than two groups: no pipeline.
-  const int64_t min_tiles = 2 * (int64_t)std::max(1, p->ctx ? p->ctx->num_sms : 0);
+  const int64_t min_tiles = (int64_t)std::max(1, p->ctx ? p->ctx->num_sms : 0);
   double total = 0.0;
   for (int64_t q : order) total += 2.0 * p->sectors[q].M * p->sectors[q].N * p->sectors[q].K;
   int64_t tile_end = 0, gt = 0;
   double gf = 0.0;
   for (int64_t oi = 0; oi < nsec; oi++) {
     const HostSector &h = p->sectors[order[oi]];
-    const int64_t nt = ((h.M + kSplitBM - 1) / kSplitBM) * ((h.N + kSplitBM - 1) / kSplitBM);
+    const int64_t nt = ((h.M + kSplitBM - 1) / kSplitBM) * ((h.N + 2 * kSplitBM - 1) / (2 * kSplitBM));
     tile_end += nt;
     gt += nt;
     gf += 2.0 * h.M * h.N * h.K;

@@ -17,7 +17,8 @@
 //                        swizzled layout.
 // Both take the items of a range [items, items + nitems): the whole list, or one
 // sector group of the pipelined variant (its instances launched beside the split
-// GEMM are sized to share an SM with a GEMM CTA).
+// GEMM are sized to share an SM with a GEMM CTA of four slices; with more slices the
+// GEMM's rings take the shared memory, and they run where it leaves an SM idle).
 // HBM traffic per operand element: 8 bytes read twice and 2 s bytes written (the
 // staged path moves 8 bytes in and out of an FP64 sector matrix first, then reads
 // it twice).
@@ -348,8 +349,8 @@ __global__ void __launch_bounds__(kThreads, 8) split_rowmax_kernel(const SplitOp
 
 // MINB: CTAs per SM the launch bounds ask for. 5: 48 registers (five CTAs per SM,
 // as shared memory allows), the fastest alone; 6: 40
-// registers, so that one CTA fits beside a split-GEMM CTA (576 threads x 96
-// registers + 256 x 40 = 65,536; shared memory 198,912 + 34,176 bytes with the
+// registers, so that one CTA fits beside a split-GEMM CTA of four slices (576 threads x
+// 96 registers + 256 x 40 = 65,536; shared memory 198,912 + 34,176 bytes with the
 // per-CTA reserve, within the SM's 233,472), for the slicing that runs beside the
 // GEMM in the pipelined variant.
 template <int MINB>

@@ -226,11 +226,22 @@ struct SplitSector {
 };
 static_assert(sizeof(SplitSector) == 72, "SplitSector layout");
 
-// One output tile of the split GEMM: 128 rows x bn columns (bn = 128, or 64 for a
-// narrow tile; nt counts tiles of that width).
+// One output tile of the split GEMM, computed by a pair of CTAs: 256 rows of the P
+// operand (128-row tiles 2 pt and 2 pt + 1, one per CTA) times bn rows of the Q operand
+// (bn = 128, or 64 for a narrow tile; qt counts tiles of that width). P is B (columns of
+// C) and Q is A, or the other way round (swap). ks: K stages of the sector. The other
+// fields give the epilogue its tables without a look at the sector: the rows left of
+// either operand, the tile's first entries among the operands' exponents and rows or
+// columns of C (OutRow, OutCol), and the sector's table of block offsets with its row
+// length; with the dense C_q as the destination, its offset and row length (ld).
 struct SplitTile {
-  int32_t sector, mt, nt, bn;
+  int32_t sector, pt, qt;
+  int16_t bn, swap;
+  int32_t ks, np, nq, q_first;
+  int64_t p_exp, q_exp, p_rec, q_rec, base, c_off;
+  int32_t ncb, ld;
 };
+static_assert(sizeof(SplitTile) == 88, "SplitTile layout");
 
 // Accuracy check of a split-precision call, written into the workspace after the
 // column exponents (see split_check.cu):
