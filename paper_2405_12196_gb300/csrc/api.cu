@@ -213,11 +213,11 @@ static void note_capture(ytn_plan_t *p, cudaStream_t st) {
 // Workspace: WA | WB | WC (FP64 sector matrices), then for the split path
 // SA | SB (BF16 slice blocks) | EA | EB (row / column exponents) and the accuracy
 // check: EMAX | NORMSQ | REC | SECV | FLAGGED | TILE_END (see SplitRecord);
-// 256-byte aligned regions, except that EMAX follows EB and REC follows NORMSQ
-// directly so that one memset covers each pair.
+// 256-byte aligned regions, except that EMAX follows EB directly so that one memset
+// covers both; another covers NORMSQ, REC and SECV.
 struct WsLayout {
   size_t wa = 0, wb = 0, wc = 0, sa = 0, sb = 0, ea = 0, eb = 0;
-  size_t emax = 0, emax_end = 0, normsq = 0, rec = 0, rec_end = 0, secv = 0, flagged = 0, tile_end = 0;
+  size_t emax = 0, emax_end = 0, normsq = 0, rec = 0, rec_end = 0, secv = 0, secv_end = 0, flagged = 0, tile_end = 0;
   size_t item_end_a = 0, item_end_b = 0;
 };
 
@@ -250,7 +250,8 @@ static size_t workspace_layout(const ytn_plan_t *p, bool split, WsLayout &w) {
   w.rec_end = o;
   o = align256(o);
   w.secv = o;
-  o += align256(nsec * 8);
+  o += align256(nsec * 16);
+  w.secv_end = o;
   w.flagged = o;
   o += align256(nsec * 4);
   w.tile_end = o;
@@ -797,7 +798,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
       if (e == cudaSuccess) {
         PhaseTimer t(p->ctx, YTN_PHASE_SPLIT, hi);
         e = cudaMemsetAsync(ea, 0x80, w.emax_end - w.ea, hi);
-        if (e == cudaSuccess) e = cudaMemsetAsync(normsq, 0, w.rec_end - w.normsq, hi);
+        if (e == cudaSuccess) e = cudaMemsetAsync(normsq, 0, w.secv_end - w.normsq, hi);
         if (e == cudaSuccess)
           e = launch_split_blocks(p->d_sp_ops, p->d_sp_fitems, ie[0], p->d_sp_segs, a, b, ea, eb, emax, sa, sb, slices,
                                   false, hi);
@@ -832,7 +833,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
         // below every exponent (bytes 0x80: 0x80808080 as int32); the epilogue sums
         // into NORMSQ and the check counts in the record: start from zero
         e = cudaMemsetAsync(ea, 0x80, w.emax_end - w.ea, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(normsq, 0, w.rec_end - w.normsq, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(normsq, 0, w.secv_end - w.normsq, st);
         if (e == cudaSuccess) {
           if (fused)
             e = launch_split_blocks(p->d_sp_ops, p->d_sp_fitems, (int64_t)p->sp_fitems.size(), p->d_sp_segs, a, b,
@@ -860,7 +861,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
       int32_t *tile_end = reinterpret_cast<int32_t *>(ws + w.tile_end);
       int32_t *item_end_a = reinterpret_cast<int32_t *>(ws + w.item_end_a);
       int32_t *item_end_b = reinterpret_cast<int32_t *>(ws + w.item_end_b);
-      e = launch_split_check(p->d_sp_sectors, (int64_t)p->sp_sectors.size(), ea, eb, emax, normsq,
+      e = launch_split_check(p->d_sp_sectors, (int64_t)p->sp_sectors.size(), p->max_m + p->max_n, ea, eb, emax, normsq,
                              reinterpret_cast<double *>(ws + w.secv), flagged, tile_end, item_end_a, item_end_b, rec,
                              split_eta(slices), kEtaFp64, rtol, slices, p->ctx->status_dev, st);
       if (e == cudaSuccess && fused && !p->sp_sectors.empty())

@@ -12,9 +12,13 @@
 // large element and the rest far below it, or when the products cancel, the
 // scales are large against |c_ij| and the estimate grows with that ratio.
 //
-// One CTA per sector computes est_q from the exponents and the ||C_q||^2 that
-// the GEMM epilogue summed (both taken relative to the operands' largest
-// exponents, so nothing overflows). The last CTA to finish:
+// A CTA sums the scales of kRows rows of one sector's operands (both taken relative
+// to the operands' largest exponents, so nothing overflows): FP64 additions are slow on
+// this GPU, two a clock and SM, so the rows of a large sector are shared out (one CTA
+// per sector took 83 us for two sectors of 133,000 rows and columns). The last CTA to
+// finish, from these and the ||C_q||^2 that the GEMM epilogue summed, with one division
+// per sector and the lists only when a sector is flagged (a chain of latencies: square
+// roots and four prefix sums per sector made it 17 to 24 us, now 13 to 14):
 //   - lists the sectors with est_q > rtol, in sector order, with the running
 //     counts of their 64 x 64 tiles and of their gather work items (the FP64
 //     recomputation reads these lists);
@@ -27,6 +31,7 @@
 // recorded into a graph.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <climits>
 #include <cmath>
 
@@ -37,36 +42,30 @@ namespace ytn {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kRows = 4096;   // rows of A and B together that one CTA sums
 
 // 4^k for k <= 0 as an FP64 value built from its bits (0 below the normal range).
 __device__ __forceinline__ double pow4(int k) {
   return k >= -511 ? __longlong_as_double((long long)(1023 + 2 * k) << 52) : 0.0;
 }
 
-__device__ __forceinline__ double block_sum(double v, double *red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  double t = 0.0;
-#pragma unroll
-  for (int w = 0; w < kThreads / 32; w++) t += red[w];
-  return t;
+  return v;
 }
 
-__device__ __forceinline__ int block_max(int v, int *red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  int t = red[0];
-#pragma unroll
-  for (int w = 1; w < kThreads / 32; w++) t = max(t, red[w]);
-  return t;
+// This thread's share of the sum of 4^(e[i] - E) over rows [lo, hi).
+__device__ __forceinline__ double scale_sum(const int32_t *__restrict__ e, int lo, int hi, int E) {
+  double s = 0.0;
+  int i = lo + 4 * (int)threadIdx.x;
+#pragma unroll 4
+  for (; i + 4 <= hi; i += 4 * kThreads) {   // rows start on multiples of 128
+    const int4 x = *reinterpret_cast<const int4 *>(e + i);
+    s += (pow4(x.x - E) + pow4(x.y - E)) + (pow4(x.z - E) + pow4(x.w - E));
+  }
+  for (; i < hi; i++) s += pow4(e[i] - E);   // the one thread whose four rows meet hi
+  return s;
 }
 
 // Exclusive prefix sum over the block (one value per thread); returns the
@@ -96,63 +95,80 @@ __device__ __forceinline__ int block_scan(int v, int *red, int *total) {
 constexpr int kZeroExp = -1021;
 
 __global__ void __launch_bounds__(kThreads) split_check_kernel(
-    const SplitSector *__restrict__ sectors, int nsec, const int32_t *__restrict__ ea, const int32_t *__restrict__ eb,
-    const int32_t *__restrict__ emax, const float *__restrict__ normsq, double *__restrict__ secv,
+    const SplitSector *__restrict__ sectors, int nsec, int nchunk, const int32_t *__restrict__ ea,
+    const int32_t *__restrict__ eb, const int32_t *__restrict__ emax, const float *__restrict__ normsq, double *secv,
     int32_t *__restrict__ flagged, int32_t *__restrict__ tile_end, int32_t *__restrict__ item_end_a,
     int32_t *__restrict__ item_end_b, SplitRecord *rec, double eta_split, double eta_fp64, double rtol, int slices,
     int *status) {
-  __shared__ double dred[kThreads / 32];
+  __shared__ double dred[4][kThreads / 32];
   __shared__ int ired[kThreads / 32];
   __shared__ int is_last;
-  const int q = blockIdx.x, tid = threadIdx.x;
-  const SplitSector sc = sectors[q];
-  const int EA = emax[2 * q], EB = emax[2 * q + 1];
-  const bool zero = EA <= kZeroExp || EB <= kZeroExp || sc.M == 0 || sc.N == 0 || sc.K == 0;
-  double se = 0.0, sf = 0.0;
-  if (!zero) {
-    for (int i = tid; i < sc.M; i += kThreads) se += pow4(ea[sc.ea_off + i] - EA);
-    for (int j = tid; j < sc.N; j += kThreads) sf += pow4(eb[sc.eb_off + j] - EB);
+  const int q = blockIdx.x / nchunk, chunk = blockIdx.x - q * nchunk, tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
+  {
+    const SplitSector sc = sectors[q];
+    const int lo = chunk * kRows, hi = lo + kRows;   // rows of A, then of B from align4(M) on
+    const int mb = (sc.M + 3) & ~3;
+    double se = 0.0, sf = 0.0;
+    if (lo < sc.M) se = scale_sum(ea + sc.ea_off, lo, min(sc.M, hi), emax[2 * q]);
+    if (hi > mb && lo - mb < sc.N) sf = scale_sum(eb + sc.eb_off, max(0, lo - mb), min(sc.N, hi - mb), emax[2 * q + 1]);
+    se = warp_sum(se);
+    sf = warp_sum(sf);
+    if (lane == 0) {
+      if (se > 0.0) atomicAdd(secv + 2 * q, se);
+      if (sf > 0.0) atomicAdd(secv + 2 * q + 1, sf);
+    }
   }
-  se = block_sum(se, dred);
-  sf = block_sum(sf, dred);
-  if (tid == 0) secv[q] = zero ? 0.0 : (double)sc.K * se * sf;
-  // the last CTA to get here sees every sector's value
+  // the last CTA to get here sees every sector's sums
   __threadfence();
   __syncthreads();
-  if (tid == 0) is_last = atomicAdd(&rec->done_blocks, 1) == nsec - 1;
+  if (tid == 0) is_last = atomicAdd(&rec->done_blocks, 1) == (int)gridDim.x - 1;
   __syncthreads();
   if (!is_last) return;
   __threadfence();
 
+  // K_q sum_i 4^(e_i - emax_A) sum_j 4^(f_j - emax_B): 0 for a zero operand
+  auto value = [&](int s) {
+    if (emax[2 * s] <= kZeroExp || emax[2 * s + 1] <= kZeroExp) return 0.0;
+    return (double)sectors[s].K * __ldcg(secv + 2 * s) * __ldcg(secv + 2 * s + 1);
+  };
   // reference exponent: the largest emax_A + emax_B among sectors with data
   int g = INT_MIN;
   for (int s = tid; s < nsec; s += kThreads)
-    if (__ldcg(secv + s) > 0.0 || normsq[s] > 0.0f) g = max(g, emax[2 * s] + emax[2 * s + 1]);
-  g = block_max(g, ired);
-  double norm = 0.0, err_split = 0.0, err_after = 0.0, flops = 0.0, worst = 0.0;
+    if (normsq[s] > 0.0f || value(s) > 0.0) g = max(g, emax[2 * s] + emax[2 * s + 1]);
+  g = __reduce_max_sync(0xffffffffu, g);
+  if (lane == 0) ired[warp] = g;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kThreads / 32; w++) g = max(g, ired[w]);
+  const double split2 = eta_split * eta_split, after2 = eta_fp64 * eta_fp64, limit = rtol * rtol;
+  double norm = 0.0, err_split = 0.0, err_after = 0.0, worst = 0.0;   // squares
   int nflag = 0, ntile = 0, nia = 0, nib = 0;
   for (int base = 0; base < nsec; base += kThreads) {
     const int s = base + tid;
-    int flag = 0, tiles = 0, ia = 0, ib = 0;
+    int flag = 0;
     if (s < nsec) {
-      const double v = __ldcg(secv + s), n2 = (double)normsq[s];
-      double est = 0.0;
-      if (v > 0.0) est = n2 > 0.0 ? eta_split * sqrt(v / n2) : INFINITY;
-      flag = est > rtol;
+      const double v = value(s), n2 = (double)normsq[s];
+      double est = 0.0;   // squared
+      if (v > 0.0) est = n2 > 0.0 ? split2 * (v / n2) : INFINITY;
+      flag = est > limit;
       worst = fmax(worst, est);
       if (g != INT_MIN) {
         const double w = pow4(emax[2 * s] + emax[2 * s + 1] - g);
         norm += n2 * w;
-        err_split += eta_split * eta_split * v * w;
-        err_after += (flag ? eta_fp64 * eta_fp64 : eta_split * eta_split) * v * w;
+        err_split += split2 * v * w;
+        err_after += (flag ? after2 : split2) * v * w;
       }
-      if (flag) {
-        const SplitSector t = sectors[s];
-        tiles = ((t.M + 63) / 64) * ((t.N + 63) / 64);
-        ia = t.ga1 - t.ga0;
-        ib = t.gb1 - t.gb0;
-        flops += 2.0 * (double)t.M * (double)t.N * (double)t.K;
-      }
+    }
+    if (!__syncthreads_or(flag)) continue;
+    // the lists of the FP64 recomputation
+    int tiles = 0, ia = 0, ib = 0;
+    if (flag) {
+      const SplitSector t = sectors[s];
+      tiles = ((t.M + 63) / 64) * ((t.N + 63) / 64);
+      ia = t.ga1 - t.ga0;
+      ib = t.gb1 - t.gb0;
+      atomicAdd(&rec->fallback_flops, 2.0 * (double)t.M * (double)t.N * (double)t.K);
     }
     int total_flag, total_tiles, total_ia, total_ib;
     const int pos = block_scan(flag, ired, &total_flag);
@@ -170,48 +186,55 @@ __global__ void __launch_bounds__(kThreads) split_check_kernel(
     nia += total_ia;
     nib += total_ib;
   }
-  norm = block_sum(norm, dred);
-  err_split = block_sum(err_split, dred);
-  err_after = block_sum(err_after, dred);
-  flops = block_sum(flops, dred);
-  {
-    // maximum of the per-sector estimates
+  norm = warp_sum(norm);
+  err_split = warp_sum(err_split);
+  err_after = warp_sum(err_after);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) worst = fmax(worst, __shfl_xor_sync(0xffffffffu, worst, o));
-    __syncthreads();
-    if ((tid & 31) == 0) dred[tid >> 5] = worst;
-    __syncthreads();
-    for (int w = 0; w < kThreads / 32; w++) worst = fmax(worst, dred[w]);
+  for (int o = 16; o > 0; o >>= 1) worst = fmax(worst, __shfl_xor_sync(0xffffffffu, worst, o));
+  if (lane == 0) {
+    dred[0][warp] = norm;
+    dred[1][warp] = err_split;
+    dred[2][warp] = err_after;
+    dred[3][warp] = worst;
   }
+  __syncthreads();
   if (tid == 0) {
+    norm = err_split = err_after = worst = 0.0;
+    for (int w = 0; w < kThreads / 32; w++) {
+      norm += dred[0][w];
+      err_split += dred[1][w];
+      err_after += dred[2][w];
+      worst = fmax(worst, dred[3][w]);
+    }
     auto rel = [&](double e2) { return e2 > 0.0 ? (norm > 0.0 ? sqrt(e2 / norm) : INFINITY) : 0.0; };
-    rec->err_est = rel(err_after);
+    const double after = rel(err_after);
+    rec->err_est = after;
     rec->split_err_est = rel(err_split);
-    rec->max_sector_est = worst;
-    rec->fallback_flops = flops;
+    rec->max_sector_est = sqrt(worst);
     rec->rtol = rtol;
     rec->nsectors = nsec;
     rec->nfallback = nflag;
-    rec->within = rec->err_est <= rtol;
+    rec->within = after <= rtol;
     rec->slices = slices;
     __threadfence();
     rec->valid = 1;
-    if (!(rec->err_est <= rtol)) atomicCAS(status + 1, 0, 1);
+    if (!(after <= rtol)) atomicCAS(status + 1, 0, 1);
   }
 }
 
 }  // namespace
 
-cudaError_t launch_split_check(const SplitSector *sectors, int64_t nsec, const int32_t *ea, const int32_t *eb,
-                               const int32_t *emax, const float *normsq, double *secv, int32_t *flagged,
-                               int32_t *tile_end, int32_t *item_end_a, int32_t *item_end_b, SplitRecord *rec,
-                               double eta_split, double eta_fp64, double rtol, int slices, int *status,
-                               cudaStream_t stream) {
+cudaError_t launch_split_check(const SplitSector *sectors, int64_t nsec, int64_t max_rows, const int32_t *ea,
+                               const int32_t *eb, const int32_t *emax, const float *normsq, double *secv,
+                               int32_t *flagged, int32_t *tile_end, int32_t *item_end_a, int32_t *item_end_b,
+                               SplitRecord *rec, double eta_split, double eta_fp64, double rtol, int slices,
+                               int *status, cudaStream_t stream) {
   if (nsec <= 0) return cudaSuccess;
-  if (nsec > INT32_MAX) return cudaErrorInvalidValue;
-  split_check_kernel<<<(unsigned)nsec, kThreads, 0, stream>>>(sectors, (int)nsec, ea, eb, emax, normsq, secv, flagged,
-                                                              tile_end, item_end_a, item_end_b, rec, eta_split,
-                                                              eta_fp64, rtol, slices, status);
+  const int64_t nchunk = std::max<int64_t>(1, (max_rows + 4 + kRows - 1) / kRows);
+  if (nsec * nchunk > INT32_MAX) return cudaErrorInvalidValue;
+  split_check_kernel<<<(unsigned)(nsec * nchunk), kThreads, 0, stream>>>(
+      sectors, (int)nsec, (int)nchunk, ea, eb, emax, normsq, secv, flagged, tile_end, item_end_a, item_end_b, rec,
+      eta_split, eta_fp64, rtol, slices, status);
   return cudaGetLastError();
 }
 

@@ -250,10 +250,10 @@ static_assert(sizeof(SplitTile) == 88, "SplitTile layout");
 //   normsq  float [nsec]      ||C_q||_F^2 times 4^-(emax_A + emax_B), summed by the
 //                             GEMM epilogue
 //   SplitRecord               the call's totals (below)
-//   secv    double [nsec]     K_q sum_i 4^(e_i - emax_A) sum_j 4^(f_j - emax_B)
+//   secv    double [2 * nsec] sum_i 4^(e_i - emax_A) and sum_j 4^(f_j - emax_B)
 //   flagged int32 [nsec]      sectors recomputed on the FP64 path, in sector order
 //   tile_end int32 [nsec]     running count of their 64 x 64 FP64 tiles
-// emax is filled with bytes 0x80 and normsq / the record with zeros before the
+// emax is filled with bytes 0x80 and normsq / the record / secv with zeros before the
 // call's kernels run.
 struct SplitRecord {
   double err_est;          // relative Frobenius error of C after the FP64 fallback
