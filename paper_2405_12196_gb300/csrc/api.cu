@@ -85,6 +85,8 @@ static ytn_status upload(ytn_plan_t *p) {
   put_table(buf, p->sp_tiles, o_spt);
   size_t o_sptm;
   put_table(buf, p->sp_tiles_mix, o_sptm);
+  size_t o_sptp;
+  put_table(buf, p->sp_tiles_pipe, o_sptp);
   put_table(buf, p->sp_fitems, o_spfi);
   put_table(buf, p->sp_segs, o_spsg);
   p->dev_bytes = align256(buf.size()) + 256;
@@ -119,6 +121,7 @@ static ytn_status upload(ytn_plan_t *p) {
   p->d_sp_slice_items = reinterpret_cast<const SplitItem *>(d + o_sps);
   p->d_sp_sectors = reinterpret_cast<const SplitSector *>(d + o_spsec);
   p->d_sp_tiles = reinterpret_cast<const SplitTile *>(d + o_spt);
+  p->d_sp_tiles_pipe = reinterpret_cast<const SplitTile *>(d + o_sptp);
   p->d_sp_tiles_mix = reinterpret_cast<const SplitTile *>(d + o_sptm);
   p->d_sp_fitems = reinterpret_cast<const SliceItem *>(d + o_spfi);
   p->d_sp_segs = reinterpret_cast<const SliceSeg *>(d + o_spsg);
@@ -807,7 +810,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
       if (e != cudaSuccess) return cuda_fail(e, "split into slices");
       {
         PhaseTimer t(p->ctx, YTN_PHASE_GEMM, hi);
-        e = launch_gemm_split(p->d_sp_sectors, p->d_sp_tiles, te[0], sa, sb, ea, eb, emax, normsq, out, slices,
+        e = launch_gemm_split(p->d_sp_sectors, p->d_sp_tiles_pipe, te[0], sa, sb, ea, eb, emax, normsq, out, slices,
                               p->ctx->status_dev, sms, false, hi);
         // enqueued after group 0's GEMM, so that its CTAs are dispatched first
         if (e == cudaSuccess) e = cudaStreamWaitEvent(lo, ev(1), 0);
@@ -819,7 +822,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
         for (size_t g = 1; g < ngroups && e == cudaSuccess; g++) {
           e = cudaStreamWaitEvent(hi, ev(g + 1), 0);
           if (e == cudaSuccess)
-            e = launch_gemm_split(p->d_sp_sectors, p->d_sp_tiles + te[g - 1], te[g] - te[g - 1], sa, sb, ea, eb, emax,
+            e = launch_gemm_split(p->d_sp_sectors, p->d_sp_tiles_pipe + te[g - 1], te[g] - te[g - 1], sa, sb, ea, eb, emax,
                                   normsq, out, slices, p->ctx->status_dev, sms, false, hi);
         }
       }

@@ -478,12 +478,12 @@ struct ytn_plan_s {
   std::vector<ytn::SliceSeg> sp_segs;
   bool sp_fused = false;
   // pipelined fused split: the sectors in the GEMM's order cut into groups; per
-  // group the end of its tiles in sp_tiles and of its items in sp_fitems (empty:
+  // group the end of its tiles in sp_tiles_pipe and of its items in sp_fitems (empty:
   // fewer than two groups). Group g's slicing runs beside group g - 1's GEMM.
   std::vector<int64_t> sp_pipe_tile_end, sp_pipe_item_end;
   std::vector<std::array<int64_t, 4>> sec_gather_items;   // per sector: A items, B items (relative)
   std::vector<ytn::SplitSector> sp_sectors;
-  std::vector<ytn::SplitTile> sp_tiles;
+  std::vector<ytn::SplitTile> sp_tiles, sp_tiles_pipe;   // the second in sector order, for runs of sectors
   std::vector<ytn::SplitTile> sp_tiles_mix;    // with 64-wide sector tails (empty: none)
   int64_t sp_sa_bytes = 0, sp_sb_bytes = 0, sp_ea = 0, sp_eb = 0;
   // YTN_AUTO: per slice count, -1 undecided, 0 FP64, 1 split; the timings (ms)
@@ -504,7 +504,7 @@ struct ytn_plan_s {
   const ytn::SplitOperand *d_sp_ops = nullptr;
   const ytn::SplitItem *d_sp_exp_items = nullptr, *d_sp_slice_items = nullptr;
   const ytn::SplitSector *d_sp_sectors = nullptr;
-  const ytn::SplitTile *d_sp_tiles = nullptr, *d_sp_tiles_mix = nullptr;
+  const ytn::SplitTile *d_sp_tiles = nullptr, *d_sp_tiles_mix = nullptr, *d_sp_tiles_pipe = nullptr;
   // the most dims of any copy item in a range [begin, end) of `items` (selects the
   // copy kernel built for at most 4 dims), computed on first use
   std::mutex nd_mu;
