@@ -322,9 +322,10 @@ static ytn_status time_runs(cudaStream_t st, const std::vector<std::function<ytn
 }
 
 // The copy launch of items [b, e) of the plan's job table, with the kernel built for
-// the most dims those items have (cached per range: a range's items never change).
-static cudaError_t copy_range(ytn_plan_t *p, int64_t b, int64_t e, const double *src, double *dst,
-                              cudaStream_t st) {
+// the most dims those items have (cached per range: a range's items never change). Items
+// from `first` on move src2 -> dst2 instead.
+static cudaError_t copy_range(ytn_plan_t *p, int64_t b, int64_t e, const double *src, double *dst, cudaStream_t st,
+                              int64_t first = INT64_MAX, const double *src2 = nullptr, double *dst2 = nullptr) {
   int nd = kMaxCopyDims;
   if (e > b && e <= (int64_t)p->items.size()) {
     const int64_t key = (b << 32) + e;
@@ -339,7 +340,7 @@ static cudaError_t copy_range(ytn_plan_t *p, int64_t b, int64_t e, const double 
       nd = m;
     }
   }
-  return launch_copy(p->d_jobs, p->d_items + b, e - b, src, dst, st, nd);
+  return launch_copy(p->d_jobs, p->d_items + b, std::min(first, e - b), e - b, src, dst, src2, dst2, st, nd);
 }
 
 }  // namespace ytn
@@ -764,15 +765,11 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
     if (p->zero_b && (e = cudaMemsetAsync(wb, 0, (size_t)p->b_elems * 8, st)) != cudaSuccess)
       return cuda_fail(e, "memset B workspace");
     {
+      // both operands' items follow one another in the table: one launch
       PhaseTimer t(p->ctx, YTN_PHASE_GATHER_A, st);
-      e = copy_range(p, p->items_a_begin, p->items_a_end, a, wa, st);
+      e = copy_range(p, p->items_a_begin, p->items_b_end, a, wa, st, p->items_a_end - p->items_a_begin, b, wb);
     }
-    if (e != cudaSuccess) return cuda_fail(e, "gather A");
-    {
-      PhaseTimer t(p->ctx, YTN_PHASE_GATHER_B, st);
-      e = copy_range(p, p->items_b_begin, p->items_b_end, b, wb, st);
-    }
-    if (e != cudaSuccess) return cuda_fail(e, "gather B");
+    if (e != cudaSuccess) return cuda_fail(e, "gather the operands");
   }
   if (!split) {
     PhaseTimer t(p->ctx, YTN_PHASE_GEMM, st);

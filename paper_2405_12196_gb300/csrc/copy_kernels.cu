@@ -193,11 +193,16 @@ __device__ __forceinline__ void run_item(const CopyJob *__restrict__ jobs, const
 template <int MAXND>
 __global__ void __launch_bounds__(kThreads, MAXND <= 4 ? 5 : 4) copy_kernel(const CopyJob *__restrict__ jobs,
                                                                            const CopyItem *__restrict__ items,
+                                                                           unsigned first,
                                                                            const double *__restrict__ src,
-                                                                           double *__restrict__ dst) {
+                                                                           double *__restrict__ dst,
+                                                                           const double *__restrict__ src2,
+                                                                           double *__restrict__ dst2) {
   __shared__ CopyJob Js[kStageJobs];
   __shared__ double stage[kStageElems];
-  run_item<MAXND>(jobs, items[blockIdx.x], src, dst, Js, stage);
+  after_previous_kernel();
+  const bool one = blockIdx.x < first;
+  run_item<MAXND>(jobs, items[blockIdx.x], one ? src : src2, one ? dst : dst2, Js, stage);
 }
 
 // Gathers of the sectors that the split path's accuracy check flagged (FP64
@@ -214,6 +219,7 @@ __global__ void __launch_bounds__(kThreads, 4) copy_flagged_kernel(const CopyJob
                                                                    double *__restrict__ dst) {
   __shared__ CopyJob Js[kStageJobs];
   __shared__ double stage[kStageElems];
+  after_previous_kernel();
   const int nflag = rec->nfallback;
   if (nflag <= 0) return;
   const int total = item_end[nflag - 1];
@@ -238,6 +244,7 @@ __global__ void __launch_bounds__(kThreads) zero_flagged_kernel(const SectorDev 
                                                                 const int32_t *__restrict__ flagged,
                                                                 const SplitRecord *__restrict__ rec, double *wa,
                                                                 double *wb, int zero_a, int zero_b) {
+  after_previous_kernel();
   const int nflag = rec->nfallback;
   for (int k = blockIdx.x; k < nflag; k += gridDim.x) {
     const SectorDev s = sectors[flagged[k]];
@@ -264,6 +271,7 @@ __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const TraceChunk *
                                                               const double *__restrict__ src,
                                                               double *__restrict__ dst) {
   __shared__ double part[kTraceThreads];
+  after_previous_kernel();
   const TraceChunk ch = chunks[blockIdx.x];
   const TraceOut &o = outs[ch.out];
   const int ne = min(kTraceElems, o.nrest - ch.e0);
@@ -339,6 +347,7 @@ __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const TraceChunk *
 __global__ void __launch_bounds__(256) cscatter_kernel(const CScatterJob *__restrict__ jobs,
                                                        const CScatterChunk *__restrict__ chunks,
                                                        const double *__restrict__ P, double *__restrict__ C) {
+  after_previous_kernel();
   const CScatterChunk ch = chunks[blockIdx.x];
   const CScatterJob J = jobs[ch.job];
   double2 *out = reinterpret_cast<double2 *>(C) + J.dst;
@@ -370,25 +379,22 @@ cudaError_t launch_cscatter(const CScatterJob *jobs, const CScatterChunk *chunks
                             double *c, cudaStream_t stream) {
   if (nchunks <= 0) return cudaSuccess;
   if (nchunks > INT32_MAX) return cudaErrorInvalidValue;
-  cscatter_kernel<<<(unsigned)nchunks, 256, 0, stream>>>(jobs, chunks, wc, c);
-  return cudaGetLastError();
+  return launch_chained(cscatter_kernel, (unsigned)nchunks, 256, 0, stream, jobs, chunks, wc, c);
 }
 
-cudaError_t launch_copy(const CopyJob *jobs, const CopyItem *items, int64_t nitems, const double *src,
-                        double *dst, cudaStream_t stream, int max_nd) {
+cudaError_t launch_copy(const CopyJob *jobs, const CopyItem *items, int64_t first, int64_t nitems, const double *src,
+                        double *dst, const double *src2, double *dst2, cudaStream_t stream, int max_nd) {
   if (nitems <= 0) return cudaSuccess;
   if (nitems > INT32_MAX || max_nd < 1 || max_nd > kMaxCopyDims) return cudaErrorInvalidValue;
-  if (max_nd <= 4) copy_kernel<4><<<(unsigned)nitems, kThreads, 0, stream>>>(jobs, items, src, dst);
-  else copy_kernel<kMaxCopyDims><<<(unsigned)nitems, kThreads, 0, stream>>>(jobs, items, src, dst);
-  return cudaGetLastError();
+  return launch_chained(max_nd <= 4 ? copy_kernel<4> : copy_kernel<kMaxCopyDims>, (unsigned)nitems, kThreads, 0, stream,
+                        jobs, items, (unsigned)first, src, dst, src2, dst2);
 }
 
 cudaError_t launch_trace(const TraceChunk *chunks, int64_t nchunks, const TraceOut *outs,
                          const TraceContrib *contribs, const double *src, double *dst, cudaStream_t stream) {
   if (nchunks <= 0) return cudaSuccess;
   if (nchunks > INT32_MAX) return cudaErrorInvalidValue;
-  trace_kernel<<<(unsigned)nchunks, kTraceThreads, 0, stream>>>(chunks, outs, contribs, src, dst);
-  return cudaGetLastError();
+  return launch_chained(trace_kernel, (unsigned)nchunks, kTraceThreads, 0, stream, chunks, outs, contribs, src, dst);
 }
 
 cudaError_t launch_gather_flagged(const CopyJob *jobs, const CopyItem *items_a, const CopyItem *items_b,
@@ -397,10 +403,17 @@ cudaError_t launch_gather_flagged(const CopyJob *jobs, const CopyItem *items_a, 
                                   const double *a, const double *b, double *wa, double *wb, bool zero_a, bool zero_b,
                                   int num_sms, cudaStream_t stream) {
   const unsigned grid = (unsigned)std::max(1, num_sms) * 4;
-  if (zero_a || zero_b) zero_flagged_kernel<<<grid, kThreads, 0, stream>>>(sectors, flagged, rec, wa, wb, zero_a, zero_b);
-  copy_flagged_kernel<<<grid, kThreads, 0, stream>>>(jobs, items_a, sp_sectors, 0, flagged, item_end_a, rec, a, wa);
-  copy_flagged_kernel<<<grid, kThreads, 0, stream>>>(jobs, items_b, sp_sectors, 1, flagged, item_end_b, rec, b, wb);
-  return cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  if (zero_a || zero_b)
+    e = launch_chained(zero_flagged_kernel, grid, kThreads, 0, stream, sectors, flagged, rec, wa, wb, (int)zero_a,
+                       (int)zero_b);
+  if (e == cudaSuccess)
+    e = launch_chained(copy_flagged_kernel, grid, kThreads, 0, stream, jobs, items_a, sp_sectors, 0, flagged, item_end_a,
+                       rec, a, wa);
+  if (e == cudaSuccess)
+    e = launch_chained(copy_flagged_kernel, grid, kThreads, 0, stream, jobs, items_b, sp_sectors, 1, flagged, item_end_b,
+                       rec, b, wb);
+  return e;
 }
 
 }  // namespace ytn

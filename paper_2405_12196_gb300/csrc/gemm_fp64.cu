@@ -233,6 +233,7 @@ __global__ void __launch_bounds__(kThreads) gemm_fp64_kernel(const SectorDev *__
                                                              const double *__restrict__ wb, OutView out) {
   __shared__ double As[2][BK][64 + PAD];
   __shared__ double Bs[2][BK][64 + PAD];
+  after_previous_kernel();
   const GemmTile tl = tiles[blockIdx.x];
   const SectorDev s = sectors[tl.sector];
   if (tl.size == 16) gemm_tile<16>(s, tl, wa, wb, out, As, Bs);
@@ -255,6 +256,7 @@ __global__ void __launch_bounds__(kThreads) gemm_fp64_redo_kernel(const SectorDe
                                                                   const double *__restrict__ wb, OutView out) {
   __shared__ double As[2][BK][64 + PAD];
   __shared__ double Bs[2][BK][64 + PAD];
+  after_previous_kernel();
   const int nflag = rec->nfallback;
   if (nflag <= 0) return;
   const int total = tile_end[nflag - 1];
@@ -279,17 +281,15 @@ __global__ void __launch_bounds__(kThreads) gemm_fp64_redo_kernel(const SectorDe
 cudaError_t launch_gemm_fp64_redo(const SectorDev *sectors, const int32_t *flagged, const int32_t *tile_end,
                                   const SplitRecord *rec, const double *wa, const double *wb, const OutView &out,
                                   int num_sms, cudaStream_t stream) {
-  gemm_fp64_redo_kernel<<<(unsigned)std::max(1, num_sms) * 4, kThreads, 0, stream>>>(sectors, flagged, tile_end, rec,
-                                                                                    wa, wb, out);
-  return cudaGetLastError();
+  return launch_chained(gemm_fp64_redo_kernel, (unsigned)std::max(1, num_sms) * 4, kThreads, 0, stream, sectors, flagged,
+                        tile_end, rec, wa, wb, out);
 }
 
 cudaError_t launch_gemm_fp64(const SectorDev *sectors, const GemmTile *tiles, int64_t ntiles,
                              const double *wa, const double *wb, const OutView &out, cudaStream_t stream) {
   if (ntiles <= 0) return cudaSuccess;
   if (ntiles > INT32_MAX) return cudaErrorInvalidValue;
-  gemm_fp64_kernel<<<(unsigned)ntiles, kThreads, 0, stream>>>(sectors, tiles, wa, wb, out);
-  return cudaGetLastError();
+  return launch_chained(gemm_fp64_kernel, (unsigned)ntiles, kThreads, 0, stream, sectors, tiles, wa, wb, out);
 }
 
 }  // namespace ytn

@@ -466,6 +466,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   using RG = Ring<S>;
   constexpr int kLeadP = 3 * kSliceBytes, kRestP = RG::kRest * kSliceBytes;   // P bytes of a slot
   extern __shared__ uint8_t smem_raw[];
+  after_previous_kernel();
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + RG::kBytes);
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + kNumBars);
@@ -925,9 +926,10 @@ cudaError_t launch_gemm_split(const SplitSector *sectors, const SplitTile *tiles
   if (ntiles <= 0) return cudaSuccess;
   if (ntiles > INT32_MAX || slices < 4 || slices > kSlices) return cudaErrorInvalidValue;
   const int64_t pairs = std::min<int64_t>(ntiles, std::max(1, num_sms / 2));
+  cudaError_t e = cudaSuccess;
   auto launch = [&](auto kernel, int smem) {
-    kernel<<<(unsigned)(2 * pairs), kThreads, smem, stream>>>(sectors, tiles, (int)ntiles, sa, sb, ea, eb, emax, normsq,
-                                                              out, status);
+    e = launch_chained(kernel, (unsigned)(2 * pairs), kThreads, (size_t)smem, stream, sectors, tiles, (int)ntiles, sa, sb,
+                       ea, eb, emax, normsq, out, status);
   };
   switch (slices + (mixed_widths ? 8 : 0)) {
     case 4: launch(gemm_split_kernel<4, false>, Ring<4>::kSmem); break;
@@ -937,7 +939,7 @@ cudaError_t launch_gemm_split(const SplitSector *sectors, const SplitTile *tiles
     case 13: launch(gemm_split_kernel<5, true>, Ring<5>::kSmem); break;
     default: launch(gemm_split_kernel<6, true>, Ring<6>::kSmem); break;
   }
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace ytn

@@ -42,6 +42,7 @@ __global__ void __launch_bounds__(kThreads) vdot_partial_kernel(const VdotChunk 
                                                                 const double *a, const double *b,
                                                                 double *__restrict__ partials) {
   __shared__ double ws[kThreads / 32];
+  after_previous_kernel();
   const VdotChunk ch = chunks[blockIdx.x];
   double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0, t0 = 0.0, t1 = 0.0;
   for (int k = ch.first; k < ch.first + ch.count; k++) {
@@ -80,6 +81,7 @@ __global__ void __launch_bounds__(kThreads) vdot_partial_kernel(const VdotChunk 
 __global__ void __launch_bounds__(kFinalThreads) vdot_final_kernel(const double *__restrict__ partials, int n,
                                                                    double *out) {
   __shared__ double ws[kFinalThreads / 32];
+  after_previous_kernel();
   double s = 0.0;
   for (int i = threadIdx.x; i < n; i += kFinalThreads) s += partials[i];
   const double t = block_sum(s, ws);
@@ -91,17 +93,14 @@ __global__ void __launch_bounds__(kFinalThreads) vdot_final_kernel(const double 
 cudaError_t launch_vdot(const VdotChunk *chunks, int64_t nchunks, const VdotPiece *pieces, const double *a,
                         const double *b, double *partials, double *out, bool complex_data, cudaStream_t stream) {
   if (nchunks > INT32_MAX / 2) return cudaErrorInvalidValue;
-  if (nchunks > 0) {
-    if (complex_data)
-      vdot_partial_kernel<true><<<(unsigned)nchunks, kThreads, 0, stream>>>(chunks, pieces, a, b, partials);
-    else
-      vdot_partial_kernel<false><<<(unsigned)nchunks, kThreads, 0, stream>>>(chunks, pieces, a, b, partials);
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  vdot_final_kernel<<<1, kFinalThreads, 0, stream>>>(partials, (int)nchunks, out);
-  if (complex_data) vdot_final_kernel<<<1, kFinalThreads, 0, stream>>>(partials + nchunks, (int)nchunks, out + 1);
-  return cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  if (nchunks > 0)
+    e = launch_chained(complex_data ? vdot_partial_kernel<true> : vdot_partial_kernel<false>, (unsigned)nchunks, kThreads,
+                       0, stream, chunks, pieces, a, b, partials);
+  if (e == cudaSuccess) e = launch_chained(vdot_final_kernel, 1, kFinalThreads, 0, stream, partials, (int)nchunks, out);
+  if (e == cudaSuccess && complex_data)
+    e = launch_chained(vdot_final_kernel, 1, kFinalThreads, 0, stream, partials + nchunks, (int)nchunks, out + 1);
+  return e;
 }
 
 }  // namespace ytn

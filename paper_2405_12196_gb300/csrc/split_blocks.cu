@@ -301,6 +301,7 @@ __global__ void __launch_bounds__(kThreads, 8) split_rowmax_kernel(const SplitOp
                                                                    int32_t *__restrict__ emax) {
   __shared__ int rmax[kRowmaxItems][kItemRows];
   __shared__ SliceItem rec[kRowmaxItems];
+  after_previous_kernel();
   const int i0 = blockIdx.x * kRowmaxItems, ni = min(kRowmaxItems, nitems - i0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid < kRowmaxItems * kItemRows) rmax[tid / kItemRows][tid % kItemRows] = 0;
@@ -364,6 +365,7 @@ __global__ void __launch_bounds__(kThreads, MINB) split_digits_kernel(const Spli
                                                                       uint8_t *__restrict__ sa,
                                                                       uint8_t *__restrict__ sb, int s) {
   __shared__ Smem sm;
+  after_previous_kernel();
   const SliceItem it = items[blockIdx.x];
   const SplitOperand o = ops[it.op];
   const bool isA = (it.op & 1) == 0;
@@ -402,17 +404,12 @@ cudaError_t launch_split_blocks(const SplitOperand *ops, const SliceItem *items,
   if (nitems <= 0) return cudaSuccess;
   if (nitems > INT32_MAX || slices < 1 || slices > kSlices) return cudaErrorInvalidValue;
   const unsigned g0 = (unsigned)((nitems + kRowmaxItems - 1) / kRowmaxItems);
-  if (beside_gemm)
-    split_rowmax_kernel<true><<<g0, kThreads, 0, stream>>>(ops, items, (int)nitems, segs, a, b, ea, eb, emax);
-  else
-    split_rowmax_kernel<false><<<g0, kThreads, 0, stream>>>(ops, items, (int)nitems, segs, a, b, ea, eb, emax);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (beside_gemm)
-    split_digits_kernel<6><<<(unsigned)nitems, kThreads, 0, stream>>>(ops, items, segs, a, b, ea, eb, sa, sb, slices);
-  else
-    split_digits_kernel<5><<<(unsigned)nitems, kThreads, 0, stream>>>(ops, items, segs, a, b, ea, eb, sa, sb, slices);
-  return cudaGetLastError();
+  cudaError_t e = launch_chained(beside_gemm ? split_rowmax_kernel<true> : split_rowmax_kernel<false>, g0, kThreads, 0,
+                                 stream, ops, items, (int)nitems, segs, a, b, ea, eb, emax);
+  if (e == cudaSuccess)
+    e = launch_chained(beside_gemm ? split_digits_kernel<6> : split_digits_kernel<5>, (unsigned)nitems, kThreads, 0, stream,
+                       ops, items, segs, a, b, ea, eb, sa, sb, slices);
+  return e;
 }
 
 }  // namespace ytn

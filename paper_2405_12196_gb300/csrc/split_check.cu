@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(kThreads) split_check_kernel(
   __shared__ double dred[4][kThreads / 32];
   __shared__ int ired[kThreads / 32];
   __shared__ int is_last;
+  after_previous_kernel();
   const int q = blockIdx.x / nchunk, chunk = blockIdx.x - q * nchunk, tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
   {
@@ -232,10 +233,9 @@ cudaError_t launch_split_check(const SplitSector *sectors, int64_t nsec, int64_t
   if (nsec <= 0) return cudaSuccess;
   const int64_t nchunk = std::max<int64_t>(1, (max_rows + 4 + kRows - 1) / kRows);
   if (nsec * nchunk > INT32_MAX) return cudaErrorInvalidValue;
-  split_check_kernel<<<(unsigned)(nsec * nchunk), kThreads, 0, stream>>>(
-      sectors, (int)nsec, (int)nchunk, ea, eb, emax, normsq, secv, flagged, tile_end, item_end_a, item_end_b, rec,
-      eta_split, eta_fp64, rtol, slices, status);
-  return cudaGetLastError();
+  return launch_chained(split_check_kernel, (unsigned)(nsec * nchunk), kThreads, 0, stream, sectors, (int)nsec, (int)nchunk,
+                        ea, eb, emax, normsq, secv, flagged, tile_end, item_end_a, item_end_b, rec, eta_split, eta_fp64,
+                        rtol, slices, status);
 }
 
 }  // namespace ytn

@@ -42,6 +42,7 @@ __global__ void __launch_bounds__(256) split_exp_kernel(const SplitOperand *__re
                                                         const double *__restrict__ wb,
                                                         int32_t *__restrict__ ea, int32_t *__restrict__ eb,
                                                         int32_t *__restrict__ emax) {
+  after_previous_kernel();
   const SplitItem it = items[blockIdx.x];
   const SplitOperand o = ops[it.op];
   const bool isA = (it.op & 1) == 0;
@@ -103,6 +104,7 @@ __global__ void __launch_bounds__(256, 6) split_slice_kernel(const SplitOperand 
                                                           int s) {
   __shared__ unsigned long long tile[kSplitBM][kSplitBK + 1];
   __shared__ int rexp[kSplitBM];
+  after_previous_kernel();
   const SplitItem it = items[blockIdx.x];
   const SplitOperand o = ops[it.op];
   const bool isA = (it.op & 1) == 0;
@@ -153,11 +155,12 @@ cudaError_t launch_split_prep(const SplitOperand *ops, const SplitItem *exp_item
                               int32_t *ea, int32_t *eb, int32_t *emax, uint8_t *sa, uint8_t *sb, int slices,
                               cudaStream_t stream) {
   if (nexp > INT32_MAX || nslice > INT32_MAX || slices < 1 || slices > kSlices) return cudaErrorInvalidValue;
-  if (nexp > 0) split_exp_kernel<<<(unsigned)nexp, 256, 0, stream>>>(ops, exp_items, wa, wb, ea, eb, emax);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (nslice > 0) split_slice_kernel<<<(unsigned)nslice, 256, 0, stream>>>(ops, slice_items, wa, wb, ea, eb, sa, sb, slices);
-  return cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  if (nexp > 0) e = launch_chained(split_exp_kernel, (unsigned)nexp, 256, 0, stream, ops, exp_items, wa, wb, ea, eb, emax);
+  if (e == cudaSuccess && nslice > 0)
+    e = launch_chained(split_slice_kernel, (unsigned)nslice, 256, 0, stream, ops, slice_items, wa, wb, ea, eb, sa, sb,
+                       slices);
+  return e;
 }
 
 }  // namespace ytn
