@@ -773,7 +773,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
   }
   if (!split) {
     PhaseTimer t(p->ctx, YTN_PHASE_GEMM, st);
-    e = launch_gemm_fp64(p->d_sectors, p->d_tiles, (int64_t)p->tiles.size(), wa, wb, out, st);
+    e = launch_gemm_fp64(p->d_sectors, p->d_tiles, (int64_t)p->tiles.size(), wa, wb, out, p->outer, st);
     if (e != cudaSuccess) return cuda_fail(e, "grouped FP64 GEMM");
   } else {
     int32_t *ea = reinterpret_cast<int32_t *>(ws + w.ea), *eb = reinterpret_cast<int32_t *>(ws + w.eb);

@@ -17,7 +17,7 @@
 // with K <= 2 (double layers contracted over a physical leg: one element per charge)
 // take plain multiply-adds, one per K, instead of a DMMA step of 4. The Z2 D = 8
 // double layer (2 sectors of 2048 x 2048 x 1) took 260 us with K padded to 16 and
-// takes 50 us.
+// takes 38 us (gemm_outer_kernel).
 //
 // The epilogue writes C's blocks directly through the planner's row, column and block
 // tables (OutView), or the dense C_q of the workspace when a scatter follows.
@@ -186,36 +186,40 @@ __device__ __forceinline__ void gemm_tile(const SectorDev &s, const GemmTile &tl
   store_tile_out<NB>(s, tl.sector, out, acc, m0 + wm + (lane >> 2), n0 + wn + 2 * (lane & 3));
 }
 
-// Sectors with K <= 2: one 64 x 64 tile by 128 threads, thread t the rows of its half
-// (t / 64, every second one) at column t % 64, so that the stores of a warp run along
-// the columns. The products are summed in the order of k, as the DMMA steps do.
+// Sectors with K <= 2: one tile of 64 rows x COLS columns by 2 COLS threads, thread t the
+// rows of its half (t / COLS, every second one) at column t % COLS, so that the stores of
+// a warp run along the columns. The products are summed in the order of k, as the DMMA
+// steps do.
 constexpr int kOuterK = 2;
 
+template <int COLS>
 __device__ __forceinline__ void outer_tile(const SectorDev &s, const GemmTile &tl, const double *__restrict__ wa,
                                            const double *__restrict__ wb, const OutView &out, double (*As)[64],
                                            OutRow *rows) {
   const int M = s.M, N = s.N, K = s.K, t = threadIdx.x;
-  const int m0 = tl.mt * 64, n = tl.nt * 64 + (t & 63);
+  const int m0 = tl.mt * 64, n = tl.nt * COLS + (t & (COLS - 1));
   const int nr = min(64, M - m0);
   const bool direct = out.sec != nullptr;
   const SectorOut so = direct ? out.sec[tl.sector] : SectorOut{};
-  for (int e = t; e < nr * K; e += kThreads) {
+  for (int e = t; e < nr * K; e += 2 * COLS) {
     const int r = e / K, k = e - r * K;
     As[k][r] = wa[s.a_off + (s.a_kmajor ? (int64_t)(m0 + r) * K + k : (int64_t)k * M + m0 + r)];
   }
   if (t < nr) rows[t] = direct ? out.rows[so.rows + m0 + t] : OutRow{0, m0 + t};
+  double b[kOuterK];
+  OutCol col{0, n, N, 0};
+  if (n < N) {
+#pragma unroll
+    for (int k = 0; k < kOuterK; k++)
+      b[k] = k < K ? __ldg(wb + s.b_off + (s.b_kmajor ? (int64_t)n * K + k : (int64_t)k * N + n)) : 0.0;
+    if (direct) col = out.cols[so.cols + n];
+  }
   __syncthreads();
   if (n >= N) return;
-  double b[kOuterK];
-#pragma unroll
-  for (int k = 0; k < kOuterK; k++)
-    b[k] = k < K ? __ldg(wb + s.b_off + (s.b_kmajor ? (int64_t)n * K + k : (int64_t)k * N + n)) : 0.0;
-  const OutCol col = direct ? out.cols[so.cols + n] : OutCol{0, n, N, 0};
-  int blk = -1;
+  int blk = direct ? -1 : 0;
   int64_t base = s.c_off;
-  if (!direct) blk = 0;
 #pragma unroll 4
-  for (int r = t >> 6; r < nr; r += 2) {
+  for (int r = t / COLS; r < nr; r += 2) {
     const OutRow row = rows[r];
     if (row.blk != blk) {
       blk = row.blk;
@@ -225,6 +229,22 @@ __device__ __forceinline__ void outer_tile(const SectorDev &s, const GemmTile &t
     if (K > 1) v = fma(As[1][r], b[1], v);
     if (base >= 0) out.c[base + (int64_t)row.idx * col.len + col.idx] = v;
   }
+}
+
+// Plans of such sectors only (tiles of 64 x 128, 128 the tile's size): small shared
+// memory, so that eight CTAs per SM hide the loads at a tile's start. Bound by the FP64
+// multiplications, 16 clocks a warp and SM; the Z2 D = 8 double layer (8.4e6 elements,
+// 67 MB) 38 us, 50 us as 64 x 64 tiles among the DMMA kernel's.
+__global__ void __launch_bounds__(256) gemm_outer_kernel(const SectorDev *__restrict__ sectors,
+                                                         const GemmTile *__restrict__ tiles,
+                                                         const double *__restrict__ wa, const double *__restrict__ wb,
+                                                         OutView out) {
+  __shared__ double As[kOuterK][64];
+  __shared__ OutRow rows[64];
+  after_previous_kernel();
+  const GemmTile tl = tiles[blockIdx.x];
+  const SectorDev s = sectors[tl.sector];
+  outer_tile<128>(s, tl, wa, wb, out, As, rows);
 }
 
 __global__ void __launch_bounds__(kThreads) gemm_fp64_kernel(const SectorDev *__restrict__ sectors,
@@ -239,7 +259,7 @@ __global__ void __launch_bounds__(kThreads) gemm_fp64_kernel(const SectorDev *__
   if (tl.size == 16) gemm_tile<16>(s, tl, wa, wb, out, As, Bs);
   else if (tl.size == 32) gemm_tile<32>(s, tl, wa, wb, out, As, Bs);
   else if (s.K <= kOuterK)
-    outer_tile(s, tl, wa, wb, out, reinterpret_cast<double(*)[64]>(&As[0][0][0]),
+    outer_tile<64>(s, tl, wa, wb, out, reinterpret_cast<double(*)[64]>(&As[0][0][0]),
                reinterpret_cast<OutRow *>(&Bs[0][0][0]));
   else gemm_tile<64>(s, tl, wa, wb, out, As, Bs);
 }
@@ -286,9 +306,10 @@ cudaError_t launch_gemm_fp64_redo(const SectorDev *sectors, const int32_t *flagg
 }
 
 cudaError_t launch_gemm_fp64(const SectorDev *sectors, const GemmTile *tiles, int64_t ntiles,
-                             const double *wa, const double *wb, const OutView &out, cudaStream_t stream) {
+                             const double *wa, const double *wb, const OutView &out, bool outer, cudaStream_t stream) {
   if (ntiles <= 0) return cudaSuccess;
   if (ntiles > INT32_MAX) return cudaErrorInvalidValue;
+  if (outer) return launch_chained(gemm_outer_kernel, (unsigned)ntiles, 256, 0, stream, sectors, tiles, wa, wb, out);
   return launch_chained(gemm_fp64_kernel, (unsigned)ntiles, kThreads, 0, stream, sectors, tiles, wa, wb, out);
 }
 

@@ -55,9 +55,9 @@ cudaError_t launch_vdot(const VdotChunk *chunks, int64_t nchunks, const VdotPiec
                         const double *b, double *partials, double *out, bool complex_data, cudaStream_t stream);
 
 // Grouped FP64 GEMM (DMMA) over the tile list: C_q = A_q B_q, into C's blocks or the
-// dense C_q (see OutView).
+// dense C_q (see OutView). outer: every sector has K <= 2, tiles of 64 x 128.
 cudaError_t launch_gemm_fp64(const SectorDev *sectors, const GemmTile *tiles, int64_t ntiles,
-                             const double *wa, const double *wb, const OutView &out, cudaStream_t stream);
+                             const double *wa, const double *wb, const OutView &out, bool outer, cudaStream_t stream);
 
 // Split-precision path: row exponents and BF16 slices of every sector operand.
 // Staged path (from the FP64 sector matrices wa, wb): row exponents (ea, eb;

@@ -1205,7 +1205,9 @@ ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int n
   // largest of 64, 32, 16 whose tile is at most a quarter of an SM's share of the
   // plan's work (17 ragged sectors up to 251 x 188 x 188: 64 x 64 tiles kept 64 of 152
   // SMs busy, 229 us; 16 x 16 62 us).
+  // Plans with K <= 2 in every sector take a kernel of their own.
   p->tiles.clear();
+  p->outer = p->max_k <= 2;
   double work = 0.0;
   for (const HostSector &h : p->sectors) work += (double)((h.M + 7) / 8 * 8) * ((h.N + 7) / 8 * 8) * h.K;
   const double share = work / std::max(1, p->ctx ? p->ctx->num_sms : 0);
@@ -1213,7 +1215,8 @@ ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int n
     const int64_t M = p->sectors[si].M, N = p->sectors[si].N;
     int T = 64;
     while (T > 16 && 4.0 * T * T * p->sectors[si].K > share) T /= 2;
-    const int64_t mt = (M + T - 1) / T, nt = (N + T - 1) / T;
+    if (p->outer) T = 128;
+    const int64_t mt = (M + std::min(T, 64) - 1) / std::min(T, 64), nt = (N + T - 1) / T;
     for (int64_t i = 0; i < mt; i++)
       for (int64_t j = 0; j < nt; j++) p->tiles.push_back({(int32_t)si, (int32_t)i, (int32_t)j, T});
   }

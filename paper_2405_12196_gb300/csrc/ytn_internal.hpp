@@ -110,7 +110,7 @@ struct OutView {
 struct GemmTile {
   int32_t sector;
   int32_t mt, nt;   // tile coordinates in units of `size`
-  int32_t size;     // tile edge: 64, 32 or 16
+  int32_t size;     // tile edge: 64, 32 or 16; 128: 64 rows x 128 columns (outer products)
 };
 
 // Trace: one output block, fed by ncontrib contributing input blocks with nterms
@@ -419,6 +419,7 @@ struct ytn_plan_s {
   std::vector<ytn::HostSector> sectors;
   std::vector<ytn::SectorDev> sectors_dev;
   std::vector<ytn::GemmTile> tiles;
+  bool outer = false;   // every sector has K <= 2 and the tiles are 64 x 128
   bool zero_a = false, zero_b = false;
   bool a_kmajor = true, b_kmajor = false;
   int64_t a_elems = 0, b_elems = 0, c_elems = 0;
