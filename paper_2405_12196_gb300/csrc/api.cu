@@ -216,11 +216,11 @@ static void note_capture(ytn_plan_t *p, cudaStream_t st) {
 // Workspace: WA | WB | WC (FP64 sector matrices), then for the split path
 // SA | SB (BF16 slice blocks) | EA | EB (row / column exponents) and the accuracy
 // check: EMAX | NORMSQ | REC | SECV | FLAGGED | TILE_END (see SplitRecord);
-// 256-byte aligned regions, except that EMAX follows EB directly so that one memset
-// covers both; another covers NORMSQ, REC and SECV.
+// 256-byte aligned regions, except that EMAX follows EB directly; one memset covers EA to
+// SECV.
 struct WsLayout {
   size_t wa = 0, wb = 0, wc = 0, sa = 0, sb = 0, ea = 0, eb = 0;
-  size_t emax = 0, emax_end = 0, normsq = 0, rec = 0, rec_end = 0, secv = 0, secv_end = 0, flagged = 0, tile_end = 0;
+  size_t emax = 0, normsq = 0, rec = 0, rec_end = 0, secv = 0, secv_end = 0, flagged = 0, tile_end = 0;
   size_t item_end_a = 0, item_end_b = 0;
 };
 
@@ -244,7 +244,6 @@ static size_t workspace_layout(const ytn_plan_t *p, bool split, WsLayout &w) {
   const size_t nsec = p->sp_sectors.size();
   w.emax = o;
   o += 2 * nsec * 4;
-  w.emax_end = o;
   o = align256(o);
   w.normsq = o;
   o += align256(nsec * 4);
@@ -797,8 +796,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
       if (e == cudaSuccess) e = cudaStreamWaitEvent(hi, ev(0), 0);
       if (e == cudaSuccess) {
         PhaseTimer t(p->ctx, YTN_PHASE_SPLIT, hi);
-        e = cudaMemsetAsync(ea, 0x80, w.emax_end - w.ea, hi);
-        if (e == cudaSuccess) e = cudaMemsetAsync(normsq, 0, w.secv_end - w.normsq, hi);
+        e = cudaMemsetAsync(ea, 0, w.secv_end - w.ea, hi);
         if (e == cudaSuccess)
           e = launch_split_blocks(p->d_sp_ops, p->d_sp_fitems, ie[0], p->d_sp_segs, a, b, ea, eb, emax, sa, sb, slices,
                                   false, hi);
@@ -829,11 +827,9 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
     } else {
       {
         PhaseTimer t(p->ctx, YTN_PHASE_SPLIT, st);
-        // the exponent kernels max-combine into EA, EB and EMAX: start from a value
-        // below every exponent (bytes 0x80: 0x80808080 as int32); the epilogue sums
-        // into NORMSQ and the check counts in the record: start from zero
-        e = cudaMemsetAsync(ea, 0x80, w.emax_end - w.ea, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(normsq, 0, w.secv_end - w.normsq, st);
+        // the exponent kernels max-combine into EA, EB and EMAX, the epilogue sums into
+        // NORMSQ, the check into SECV and counts in the record: all start from zero
+        e = cudaMemsetAsync(ea, 0, w.secv_end - w.ea, st);
         if (e == cudaSuccess) {
           if (fused)
             e = launch_split_blocks(p->d_sp_ops, p->d_sp_fitems, (int64_t)p->sp_fitems.size(), p->d_sp_segs, a, b,

@@ -206,35 +206,42 @@ __global__ void __launch_bounds__(kThreads, MAXND <= 4 ? 5 : 4) copy_kernel(cons
 }
 
 // Gathers of the sectors that the split path's accuracy check flagged (FP64
-// fallback): a persistent grid walks the flagged sectors' work items (each
-// sector's items are [first[q], first[q] + count), the running counts over the
-// flagged sectors in item_end). With no flagged sector every CTA returns at once.
+// fallback): a persistent grid, even CTAs for A and odd ones for B, walks the flagged
+// sectors' work items (each sector's items are [first[q], first[q] + count), the
+// running counts over the flagged sectors in item_end). With no flagged sector every
+// CTA returns at once.
+struct FlaggedGather {
+  const CopyItem *items;
+  const int32_t *item_end;
+  const double *src;
+  double *dst;
+};
+
 __global__ void __launch_bounds__(kThreads, 4) copy_flagged_kernel(const CopyJob *__restrict__ jobs,
-                                                                   const CopyItem *__restrict__ items,
-                                                                   const SplitSector *__restrict__ sectors, int which,
+                                                                   const SplitSector *__restrict__ sectors,
                                                                    const int32_t *__restrict__ flagged,
-                                                                   const int32_t *__restrict__ item_end,
                                                                    const SplitRecord *__restrict__ rec,
-                                                                   const double *__restrict__ src,
-                                                                   double *__restrict__ dst) {
+                                                                   FlaggedGather ga, FlaggedGather gb) {
   __shared__ CopyJob Js[kStageJobs];
   __shared__ double stage[kStageElems];
   after_previous_kernel();
   const int nflag = rec->nfallback;
   if (nflag <= 0) return;
-  const int total = item_end[nflag - 1];
-  for (int t = blockIdx.x; t < total; t += gridDim.x) {
+  const bool isA = (blockIdx.x & 1) == 0;
+  const FlaggedGather g = isA ? ga : gb;
+  const int total = g.item_end[nflag - 1];
+  for (int t = blockIdx.x >> 1; t < total; t += gridDim.x >> 1) {
     int lo = 0, hi = nflag - 1;   // first flagged sector whose items end after t
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
-      if (item_end[mid] > t) hi = mid;
+      if (g.item_end[mid] > t) hi = mid;
       else lo = mid + 1;
     }
     const SplitSector &sc = sectors[flagged[lo]];
-    const int first = which == 0 ? sc.ga0 : sc.gb0;
-    const int local = t - (lo > 0 ? item_end[lo - 1] : 0);
+    const int first = isA ? sc.ga0 : sc.gb0;
+    const int local = t - (lo > 0 ? g.item_end[lo - 1] : 0);
     __syncthreads();   // the previous item's shared memory is no longer read
-    run_item<kMaxCopyDims>(jobs, items[first + local], src, dst, Js, stage);
+    run_item<kMaxCopyDims>(jobs, g.items[first + local], g.src, g.dst, Js, stage);
   }
 }
 
@@ -408,11 +415,8 @@ cudaError_t launch_gather_flagged(const CopyJob *jobs, const CopyItem *items_a, 
     e = launch_chained(zero_flagged_kernel, grid, kThreads, 0, stream, sectors, flagged, rec, wa, wb, (int)zero_a,
                        (int)zero_b);
   if (e == cudaSuccess)
-    e = launch_chained(copy_flagged_kernel, grid, kThreads, 0, stream, jobs, items_a, sp_sectors, 0, flagged, item_end_a,
-                       rec, a, wa);
-  if (e == cudaSuccess)
-    e = launch_chained(copy_flagged_kernel, grid, kThreads, 0, stream, jobs, items_b, sp_sectors, 1, flagged, item_end_b,
-                       rec, b, wb);
+    e = launch_chained(copy_flagged_kernel, grid, kThreads, 0, stream, jobs, sp_sectors, flagged, rec,
+                       FlaggedGather{items_a, item_end_a, a, wa}, FlaggedGather{items_b, item_end_b, b, wb});
   return e;
 }
 

@@ -834,7 +834,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       // issuer waits for what exceeds the first chunk of the next tile.
       const int pref = __ldg(emax + 2 * tl.sector + (swap ? 0 : 1)), qref = __ldg(emax + 2 * tl.sector + (swap ? 1 : 0));
       const int64_t step = swap ? 1 : len;
-      const int e0 = ep + qref - 40;
+      const int e0 = ep + qref - 2 * kExpBias - 40;
       uq = max(uq - qref, -4096);
       // full width, few blocks, every result normal and every sum below 2^51?
       const int umin = __reduce_min_sync(0xffffffffu, lane < nq ? uq : 0);

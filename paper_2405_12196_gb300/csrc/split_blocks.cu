@@ -280,7 +280,7 @@ __device__ __forceinline__ void rowmax_units(int *rmax, const SliceSeg &g, int u
 }
 
 // Row maxima of the biased exponent over each item's elements, combined over the
-// row's items into its scale exponent (E = max - 1021, so that |x| < 2^(E - 1))
+// row's items into E (the scale exponent is e = E - kExpBias, so that |x| < 2^(e - 1))
 // with atomicMax, and into the operand's largest. Rows without elements in the item
 // count as 0 (as zeros do). No staging: the elements are read straight into
 // registers. A CTA takes two consecutive items (their records and segment tables
@@ -339,8 +339,8 @@ __global__ void __launch_bounds__(kThreads, 8) split_rowmax_kernel(const SplitOp
     int mine = INT_MIN;
     if (row < o.rows) {
       const int r = rmax[warp][lane];
-      atomicMax((isA ? ea : eb) + o.exp_off + row, r - 1021);
-      mine = r - 1021;
+      atomicMax((isA ? ea : eb) + o.exp_off + row, r);
+      mine = r;
     }
 #pragma unroll
     for (int s = 16; s > 0; s >>= 1) mine = max(mine, __shfl_xor_sync(0xffffffffu, mine, s));
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kThreads, MINB) split_digits_kernel(const Spli
   const bool isA = (it.op & 1) == 0;
   const int tid = threadIdx.x;
   const int row0 = it.rt * kSplitBM + it.quarter * kItemRows;
-  if (tid < kItemRows) sm.rexp[tid] = row0 + tid < o.rows ? ((isA ? ea : eb) + o.exp_off)[row0 + tid] : -1021;
+  if (tid < kItemRows) sm.rexp[tid] = (row0 + tid < o.rows ? ((isA ? ea : eb) + o.exp_off)[row0 + tid] : 0) - kExpBias;
   load_item(sm, it, segs, isA ? a : b);
   uint8_t *S = (isA ? sa : sb) + o.slice_off;
   // tasks: (stage, row, 16-byte chunk), a warp covering 8 rows of one stage (512

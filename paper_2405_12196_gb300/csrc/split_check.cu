@@ -91,9 +91,6 @@ __device__ __forceinline__ int block_scan(int v, int *red, int *total) {
   return before + x - v;
 }
 
-// A zero operand (every exponent at the zero-row value) gives an exact zero product.
-constexpr int kZeroExp = -1021;
-
 __global__ void __launch_bounds__(kThreads) split_check_kernel(
     const SplitSector *__restrict__ sectors, int nsec, int nchunk, const int32_t *__restrict__ ea,
     const int32_t *__restrict__ eb, const int32_t *__restrict__ emax, const float *__restrict__ normsq, double *secv,
@@ -130,7 +127,7 @@ __global__ void __launch_bounds__(kThreads) split_check_kernel(
 
   // K_q sum_i 4^(e_i - emax_A) sum_j 4^(f_j - emax_B): 0 for a zero operand
   auto value = [&](int s) {
-    if (emax[2 * s] <= kZeroExp || emax[2 * s + 1] <= kZeroExp) return 0.0;
+    if (emax[2 * s] <= 0 || emax[2 * s + 1] <= 0) return 0.0;
     return (double)sectors[s].K * __ldcg(secv + 2 * s) * __ldcg(secv + 2 * s + 1);
   };
   // reference exponent: the largest emax_A + emax_B among sectors with data

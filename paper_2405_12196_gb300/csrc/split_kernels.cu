@@ -30,10 +30,10 @@ namespace ytn {
 
 namespace {
 
-// Row exponents: e_r = maxE - 1021 over the row (maxE = largest biased exponent,
-// 0 for a zero row). An item covers 128 rows and up to 256 of K; its per-row
+// Row exponents: E_r = maxE, the largest biased exponent of the row (0 for a zero row),
+// so that e_r = E_r - kExpBias. An item covers 128 rows and up to 256 of K; its per-row
 // maxima are combined into E with atomicMax (exact and order-independent), E
-// having been set below every exponent beforehand. Rows past the operand are
+// having been zeroed beforehand. Rows past the operand are
 // left alone (no kernel reads them). The item's largest exponent also goes into
 // emax[op], the operand's largest (the reference scale of the accuracy check).
 __global__ void __launch_bounds__(256) split_exp_kernel(const SplitOperand *__restrict__ ops,
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(256) split_exp_kernel(const SplitOperand *__re
       for (int k = k_lo + lane; k < k_hi; k += 32) m = max(m, biased_exp(__ldg(row + k)));
 #pragma unroll
       for (int s = 16; s > 0; s >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, s));
-      if (lane == 0) atomicMax(E + r, m - 1021);
+      if (lane == 0) atomicMax(E + r, m);
       mine = max(mine, m);
     }
   } else {
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(256) split_exp_kernel(const SplitOperand *__re
     red[half][rr] = m;
     mine = m;
     __syncthreads();
-    if (tid < kSplitBM && r0 + tid < o.rows) atomicMax(E + r0 + tid, max(red[0][tid], red[1][tid]) - 1021);
+    if (tid < kSplitBM && r0 + tid < o.rows) atomicMax(E + r0 + tid, max(red[0][tid], red[1][tid]));
   }
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) mine = max(mine, __shfl_xor_sync(0xffffffffu, mine, s));
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(256) split_exp_kernel(const SplitOperand *__re
     int m = wmax[0];
 #pragma unroll
     for (int w = 1; w < 8; w++) m = max(m, wmax[w]);
-    atomicMax(emax + it.op, m - 1021);
+    atomicMax(emax + it.op, m);
   }
 }
 
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(256, 6) split_slice_kernel(const SplitOperand 
   uint8_t *S = (isA ? sa : sb) + o.slice_off;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r0 = it.rt * kSplitBM;
-  if (tid < kSplitBM) rexp[tid] = r0 + tid < o.rows ? E[r0 + tid] : -1021;
+  if (tid < kSplitBM) rexp[tid] = (r0 + tid < o.rows ? E[r0 + tid] : 0) - kExpBias;
   for (int kt = it.kt0; kt < it.kt0 + it.nkt; kt++) {
     const int k0 = kt * kSplitBK;
     __syncthreads();

@@ -165,6 +165,10 @@ constexpr int kSlices = 6;                 // slices stored per operand
 constexpr int kSliceBytes = kSplitBM * kSplitBK * 2;         // 8192
 constexpr int kBlockBytes = kSlices * kSliceBytes;           // 49152
 
+// Row exponents are kept as the row's largest biased FP64 exponent E (0 for a zero row,
+// and before any element is seen); the row's scale is 2^(E - kExpBias).
+constexpr int kExpBias = 1021;
+
 // One operand (A rows = M, or B rows = N) of one sector, for the split kernels.
 struct SplitOperand {
   int64_t src_off;     // element offset of the FP64 sector matrix in its workspace
@@ -253,8 +257,7 @@ static_assert(sizeof(SplitTile) == 88, "SplitTile layout");
 //   secv    double [2 * nsec] sum_i 4^(e_i - emax_A) and sum_j 4^(f_j - emax_B)
 //   flagged int32 [nsec]      sectors recomputed on the FP64 path, in sector order
 //   tile_end int32 [nsec]     running count of their 64 x 64 FP64 tiles
-// emax is filled with bytes 0x80 and normsq / the record / secv with zeros before the
-// call's kernels run.
+// All of them, and the exponents before them, are zeroed before the call's kernels run.
 struct SplitRecord {
   double err_est;          // relative Frobenius error of C after the FP64 fallback
   double split_err_est;    // the same for the split products alone (no fallback)
