@@ -115,38 +115,69 @@ struct Stepper {
   }
 };
 
+// The addresses along one side of a block: of index i, i + 1, ... (merged to one dim: a
+// constant stride, an addition per step).
+template <int ND>
+struct Walk {
+  Stepper<ND> w;
+  const double *base;
+  __device__ __forceinline__ void start(const double *b, int i, const int32_t *e, const int64_t *s) {
+    base = b;
+    w.start(i, e, s);
+  }
+  __device__ __forceinline__ const double *at() const { return base + w.off; }
+  __device__ __forceinline__ void step() { w.step(); }
+};
+template <>
+struct Walk<0> {
+  const double *p;
+  __device__ __forceinline__ void start(const double *b, int, const int32_t *, const int64_t *) { p = b; }
+  __device__ __forceinline__ const double *at() const { return p; }
+  __device__ __forceinline__ void step() {}
+};
+template <>
+struct Walk<1> {
+  const double *p;
+  int64_t st;
+  __device__ __forceinline__ void start(const double *b, int i, const int32_t *, const int64_t *s) {
+    st = s[0];
+    p = b + i * st;
+  }
+  __device__ __forceinline__ const double *at() const { return p; }
+  __device__ __forceinline__ void step() { p += st; }
+};
+
 // Units [u0, u1) of a segment into the tile. rfast: a unit is one column of K, the
-// lanes its rows; else a unit is one row, the lanes its K (four per lane). ND: the
-// dims of the stepped side (K when rfast, else the rows).
+// lanes its rows; else a unit is one row, the lanes its K, 32 at a time (a segment's K
+// range is mostly shorter than the item's 128: one pass per 32 instead of four copies
+// per row, most of them masked off). ND: the dims of the stepped side (K when rfast,
+// else the rows).
 template <int ND>
 __device__ __forceinline__ void load_units(Smem &sm, const SliceSeg &g, int u0, int u1, int lane,
                                            const double *__restrict__ X) {
   const int r0 = g.r0, nr = g.r1 - g.r0, k0 = g.k0, kc = g.k1 - g.k0;
   const double *base = X + g.boff;
+  Walk<ND> w;
   if (g.rfast) {
-    Stepper<ND> kw;
-    kw.start(g.kbase + u0, g.kext, g.kst);
-    const double *rb = base;
-    if (lane < nr) rb += side_offset(g.ibase + lane, g.nf, g.fext, g.fst);
-    unsigned long long *t = &sm.tile[r0 + lane][k0];
-    for (int k = u0; k < u1; k++) {
-      if (lane < nr) cp_async8(t + k, rb + kw.off);
-      kw.step();
+    if (lane < nr) {
+      w.start(base + side_offset(g.ibase + lane, g.nf, g.fext, g.fst), g.kbase + u0, g.kext, g.kst);
+      unsigned long long *t = &sm.tile[r0 + lane][k0 + u0];
+#pragma unroll 4
+      for (int k = u0; k < u1; k++) {
+        cp_async8(t++, w.at());
+        w.step();
+      }
     }
   } else {
-    int32_t ko[kItemK / 32];
-#pragma unroll
-    for (int q = 0; q < kItemK / 32; q++)
-      ko[q] = lane + 32 * q < kc ? side_offset(g.kbase + lane + 32 * q, g.nk, g.kext, g.kst) : 0;
-    Stepper<ND> rw;
-    rw.start(g.ibase + u0, g.fext, g.fst);
-    for (int r = u0; r < u1; r++) {
-      const double *rb = base + rw.off;
-      unsigned long long *t = &sm.tile[r0 + r][k0 + lane];
-#pragma unroll
-      for (int q = 0; q < kItemK / 32; q++)
-        if (lane + 32 * q < kc) cp_async8(t + 32 * q, rb + ko[q]);
-      rw.step();
+    for (int k = lane; k < kc; k += 32) {
+      w.start(base + side_offset(g.kbase + k, g.nk, g.kext, g.kst), g.ibase + u0, g.fext, g.fst);
+      unsigned long long *t = &sm.tile[r0 + u0][k0 + k];
+#pragma unroll 4
+      for (int r = u0; r < u1; r++) {
+        cp_async8(t, w.at());
+        t += kPitch;
+        w.step();
+      }
     }
   }
 }
@@ -228,53 +259,55 @@ __device__ __forceinline__ int biased_exp_at(const double *p) {
 
 // Row maxima of the biased exponent over units [u0, u1) of a segment, combined into
 // rmax (shared memory, one per row of the item). rfast: each lane keeps its row's
-// maximum over the K columns it steps through, eight loads in flight; else each row
-// is one step, its maximum reduced over the warp. ND: the dims of the stepped side.
+// maximum over the K columns it steps through, eight loads in flight; else a row is one
+// step of the lanes along K, 32 at a time, its maximum reduced over the warp, eight rows
+// in flight. A warp's part of a segment is short (some ten steps), so the last, partial
+// batch issues its loads together too, and a side merged to one dim is stepped by an
+// addition: 93 -> 89 us on the D = 12 operands (3.1e7 elements), 1283 -> 1219 us on D =
+// 20. Latency-bound all the same (loads waited for, issue slots a third busy): registers
+// for six CTAs per SM instead of eight gave 80 and 1302 us. ND: the dims of the stepped
+// side.
 template <int ND>
 __device__ __forceinline__ void rowmax_units(int *rmax, const SliceSeg &g, int u0, int u1, int lane,
                                              const double *__restrict__ X) {
+  constexpr int kBatch = 8;
   const int r0 = g.r0, nr = g.r1 - g.r0, kc = g.k1 - g.k0;
   const double *base = X + g.boff;
+  Walk<ND> w;
+  int x[kBatch];
   if (g.rfast) {
-    const bool act = lane < nr;
-    Stepper<ND> kw;
-    kw.start(g.kbase + u0, g.kext, g.kst);
-    const double *rb = base;
-    if (act) rb += side_offset(g.ibase + lane, g.nf, g.fext, g.fst);
-    int m = 0;
-    int k = u0;
-    for (; k + 8 <= u1; k += 8) {
-      int x[8];
-#pragma unroll
-      for (int q = 0; q < 8; q++) {
-        x[q] = act ? biased_exp_at(rb + kw.off) : 0;
-        kw.step();
-      }
-#pragma unroll
-      for (int q = 0; q < 8; q++) m = max(m, x[q]);
-    }
-    for (; k < u1; k++) {
-      if (act) m = max(m, biased_exp_at(rb + kw.off));
-      kw.step();
-    }
-    if (act) atomicMax(rmax + r0 + lane, m);
-  } else {
-    int32_t ko[kItemK / 32];
-#pragma unroll
-    for (int q = 0; q < kItemK / 32; q++)
-      ko[q] = lane + 32 * q < kc ? side_offset(g.kbase + lane + 32 * q, g.nk, g.kext, g.kst) : 0;
-    Stepper<ND> rw;
-    rw.start(g.ibase + u0, g.fext, g.fst);
-    for (int r = u0; r < u1; r++) {
-      const double *rb = base + rw.off;
+    if (lane < nr) {
+      w.start(base + side_offset(g.ibase + lane, g.nf, g.fext, g.fst), g.kbase + u0, g.kext, g.kst);
       int m = 0;
+      for (int k = u0; k < u1; k += kBatch) {
 #pragma unroll
-      for (int q = 0; q < kItemK / 32; q++)
-        if (lane + 32 * q < kc) m = max(m, biased_exp_at(rb + ko[q]));
+        for (int q = 0; q < kBatch; q++) {
+          x[q] = k + q < u1 ? biased_exp_at(w.at()) : 0;
+          w.step();
+        }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (lane == 0) atomicMax(rmax + r0 + r, m);
-      rw.step();
+        for (int q = 0; q < kBatch; q++) m = max(m, x[q]);
+      }
+      atomicMax(rmax + r0 + lane, m);
+    }
+  } else {
+    for (int k = 0; k < kc; k += 32) {   // uniform in the warp
+      const bool act = k + lane < kc;
+      w.start(base + (act ? side_offset(g.kbase + k + lane, g.nk, g.kext, g.kst) : 0), g.ibase + u0, g.fext, g.fst);
+      for (int r = u0; r < u1; r += kBatch) {
+#pragma unroll
+        for (int q = 0; q < kBatch; q++) {
+          x[q] = act && r + q < u1 ? biased_exp_at(w.at()) : 0;
+          w.step();
+        }
+        int mine = 0;
+#pragma unroll
+        for (int q = 0; q < kBatch; q++) {
+          const int m = __reduce_max_sync(0xffffffffu, x[q]);
+          if (lane == q) mine = m;
+        }
+        if (lane < kBatch && r + lane < u1) atomicMax(rmax + r0 + r + lane, mine);
+      }
     }
   }
 }
@@ -371,7 +404,7 @@ __global__ void __launch_bounds__(kThreads, MINB) split_digits_kernel(const Spli
   const bool isA = (it.op & 1) == 0;
   const int tid = threadIdx.x;
   const int row0 = it.rt * kSplitBM + it.quarter * kItemRows;
-  if (tid < kItemRows) sm.rexp[tid] = (row0 + tid < o.rows ? ((isA ? ea : eb) + o.exp_off)[row0 + tid] : 0) - kExpBias;
+  if (tid < kItemRows) sm.rexp[tid] = row0 + tid < o.rows ? ((isA ? ea : eb) + o.exp_off)[row0 + tid] : 0;
   load_item(sm, it, segs, isA ? a : b);
   uint8_t *S = (isA ? sa : sb) + o.slice_off;
   // tasks: (stage, row, 16-byte chunk), a warp covering 8 rows of one stage (512

@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(256, 6) split_slice_kernel(const SplitOperand 
   uint8_t *S = (isA ? sa : sb) + o.slice_off;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r0 = it.rt * kSplitBM;
-  if (tid < kSplitBM) rexp[tid] = (r0 + tid < o.rows ? E[r0 + tid] : 0) - kExpBias;
+  if (tid < kSplitBM) rexp[tid] = r0 + tid < o.rows ? E[r0 + tid] : 0;
   for (int kt = it.kt0; kt < it.kt0 + it.nkt; kt++) {
     const int k0 = kt * kSplitBK;
     __syncthreads();
