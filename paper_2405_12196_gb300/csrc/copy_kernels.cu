@@ -267,10 +267,13 @@ __global__ void __launch_bounds__(kThreads) zero_flagged_kernel(const SectorDev 
 // of the block's terms (the diagonal elements of its contributing blocks in order);
 // the workers' sums are added in a fixed order, so repeated calls give the same
 // bits. Latency-bound: the terms are single elements far apart in memory, so the
-// time is a thread's chain of loads, eight in flight; spreading the terms over 512
-// threads took the D = 16 environment's partial trace (61 output blocks, about 256
-// terms each) from 769 us (thread per output element, one CTA per block) to 24 us.
+// time is a thread's chain of loads, eight in flight, and before them its search through
+// the contributions, which are read into shared memory together when they fit. The D =
+// 16 environment's partial trace (61 output blocks, about 256 terms each): 769 us with a
+// thread per output element and a CTA per block, 24 us with the terms over 512 threads,
+// 17 us with the contributions in shared memory.
 constexpr int kTraceThreads = 512;
+constexpr int kTraceStage = 64;   // contributions kept in shared memory
 
 __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const TraceChunk *__restrict__ chunks,
                                                               const TraceOut *__restrict__ outs,
@@ -278,9 +281,18 @@ __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const TraceChunk *
                                                               const double *__restrict__ src,
                                                               double *__restrict__ dst) {
   __shared__ double part[kTraceThreads];
+  __shared__ TraceContrib staged[kTraceStage];
   after_previous_kernel();
   const TraceChunk ch = chunks[blockIdx.x];
   const TraceOut &o = outs[ch.out];
+  const TraceContrib *cs = contribs + o.first;
+  if (o.ncontrib <= kTraceStage) {
+    const int64_t *from = reinterpret_cast<const int64_t *>(cs);
+    for (int w = threadIdx.x; w < o.ncontrib * (int)(sizeof(TraceContrib) / 8); w += kTraceThreads)
+      reinterpret_cast<int64_t *>(staged)[w] = from[w];
+    cs = staged;
+    __syncthreads();
+  }
   const int ne = min(kTraceElems, o.nrest - ch.e0);
   int wide = kTraceElems;
   while (wide / 2 >= ne) wide >>= 1;
@@ -302,13 +314,13 @@ __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const TraceChunk *
       int lo = 0, hi = o.ncontrib - 1;
       while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (contribs[o.first + mid].term0 <= t0) lo = mid;
+        if (cs[mid].term0 <= t0) lo = mid;
         else hi = mid - 1;
       }
       int64_t t = t0;
       for (int c = lo; t < t1; c++) {
-        const TraceContrib &tc = contribs[o.first + c];
-        const int64_t end = c + 1 < o.ncontrib ? min(t1, contribs[o.first + c + 1].term0) : t1;
+        const TraceContrib &tc = cs[c];
+        const int64_t end = c + 1 < o.ncontrib ? min(t1, cs[c + 1].term0) : t1;
         int64_t base = tc.src_off;
 #pragma unroll
         for (int i = 0; i < kMaxCopyDims; i++)
