@@ -73,6 +73,7 @@ constexpr int kEpiWarps = 16;
 constexpr int kHalfBytes = kSliceBytes / 2;   // a CTA's half of a Q slice
 constexpr uint32_t kColE2 = 0, kColE3 = 128, kColE4 = 256, kColR = 384;
 constexpr uint32_t kMaxPolls = 1u << 26;
+constexpr int kOutGroup = 8;    // rows of Q converted without a look at C's blocks in between
 constexpr int kMaxStarts = 4;   // blocks of C among a warp's 32 rows with places read ahead
 
 // Shared memory of one CTA: two rings, since the exact products read slices 0..2 of a
@@ -845,22 +846,35 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       if (plain) {
         const double *const *next = places;
         bool put = false;
+        auto element = [&](int j) {
+          const int t = __shfl_sync(0xffffffffu, uq, j);
+          float rel;
+          const double d = j & 1 ? scaled_int(acc[j], e0 + t, t - 40, rel) : scaled_add(acc[j], e0 + t, t - 40, rel);
+          if (put) *ptr = d;
+          ptr += step;
+          ss = fmaf(rel, rel, ss);
+        };
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-          if (h == 1 && narrow) break;
+        for (int h = 0; h < 32; h += kOutGroup) {
+          if (narrow && h >= 16) break;
+          // a block starts at the group's first row or not at all, most often: then its
+          // elements follow one another without a branch and overlap
+          if (starts >> h & 1) {
+            ptr = const_cast<double *>(*next++);
+            put = ptr != nullptr;
+          }
+          if (!(starts >> h & ((1u << kOutGroup) - 2))) {
 #pragma unroll
-          for (int i = 0; i < 16; i++) {
-            const int j = 16 * h + i;
-            if (starts >> j & 1) {
-              ptr = const_cast<double *>(*next++);
-              put = ptr != nullptr;
+            for (int i = 0; i < kOutGroup; i++) element(h + i);
+          } else {
+#pragma unroll
+            for (int i = 0; i < kOutGroup; i++) {
+              if (i > 0 && (starts >> (h + i) & 1)) {
+                ptr = const_cast<double *>(*next++);
+                put = ptr != nullptr;
+              }
+              element(h + i);
             }
-            const int t = __shfl_sync(0xffffffffu, uq, j);
-            float rel;
-            const double d = j & 1 ? scaled_int(acc[j], e0 + t, t - 40, rel) : scaled_add(acc[j], e0 + t, t - 40, rel);
-            if (put) *ptr = d;
-            ptr += step;
-            ss = fmaf(rel, rel, ss);
           }
         }
         if (!in) ss = 0.0f;
