@@ -837,10 +837,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       const int64_t step = swap ? 1 : len;
       const int e0 = ep + qref - 2 * kExpBias - 40;
       uq = max(uq - qref, -4096);
-      // full width, few blocks, every result normal and every sum below 2^51?
+      // few blocks, every result normal and every sum below 2^51? (Rows past the sector have
+      // zero slices and sums; a warp at the sector's edge took the general way at first,
+      // and the whole tile waited for it.)
       const int umin = __reduce_min_sync(0xffffffffu, lane < nq ? uq : 0);
       const int lo = __reduce_min_sync(0xffffffffu, in ? e0 : 0), hi = __reduce_max_sync(0xffffffffu, in ? e0 : 0);
-      const bool plain = umin >= -80 && lo + umin > -900 && hi < 900 && tl.ks <= 252 && nq == ngroups * 4 && __popc(starts) <= kMaxStarts;
+      const bool plain = umin >= -80 && lo + umin > -900 && hi < 900 && tl.ks <= 252 && __popc(starts) <= kMaxStarts;
       float ss = 0.0f;
       double *ptr = nullptr;
       if (plain) {
@@ -850,13 +852,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           const int t = __shfl_sync(0xffffffffu, uq, j);
           float rel;
           const double d = j & 1 ? scaled_int(acc[j], e0 + t, t - 40, rel) : scaled_add(acc[j], e0 + t, t - 40, rel);
-          if (put) *ptr = d;
+          if (put && j < nq) *ptr = d;
           ptr += step;
           ss = fmaf(rel, rel, ss);
         };
 #pragma unroll
         for (int h = 0; h < 32; h += kOutGroup) {
-          if (narrow && h >= 16) break;
+          if (h >= nq) break;
           // a block starts at the group's first row or not at all, most often: then its
           // elements follow one another without a branch and overlap
           if (starts >> h & 1) {
