@@ -585,10 +585,11 @@ def measure_contraction(args, ytn, ctx, dev, cfg, world, rank, local, prec, step
     # ---- headline precision: device-resident steps
     head = measure(prec, steps, warmup, clocks=True)
     ph = phases(head)
-    # the fused split path reads A's and B's blocks in its slicing kernel (the split
-    # phase): then only the scatter of C is a data mover of its own
-    moved_elems = plan.info["moved_elems"] if "gather_a" in ph else plan.info["out_size"]
-    moved_bytes = 16.0 * moved_elems
+    # the gathers of A and B are one launch (timed as gather_a); the fused split path reads
+    # their blocks in its slicing kernels (the split phase) instead, and the GEMMs write C's
+    # blocks themselves unless C is complex (or in host memory): then a scatter does
+    moved_bytes = 16.0 * (((plan.info["moved_elems"] - plan.info["out_size"]) if "gather_a" in ph else 0)
+                          + (plan.info["out_size"] if "scatter" in ph else 0))
     mover_ms = sum(ph[k]["ms_per_call"] for k in ("gather_a", "gather_b", "scatter") if k in ph)
     out_head = dc.clone() if prec != ytn.YTN_FP64 else None
     # the data-aware accuracy record of the last timed split call (the device's own
@@ -798,12 +799,12 @@ def run_ours(args):
         # kernels of the library per timed region: one per phase call, plus the second
         # kernel of the split phase (exponents and slices, or row maxima and digits)
         # and the rest of the check phase (the FP64 recomputation; on the fused path
-        # also the gathers of the recomputed sectors, two launches; the workloads here
+        # also the gathers of the recomputed sectors, one launch; the workloads here
         # have every block of a sector, so no zero fill); the pipelined variant adds,
         # inside its GEMM phase, one GEMM and two slicing launches per further group
         "gpu_launches": int(sum(v["calls"] for v in ph.values()) + ph.get("split", {}).get("calls", 0)
                             + ph.get("check", {}).get("calls", 0)
-                            * (3 if m["head"]["res"].get("split_variant") in (1, 2) else 1)
+                            * (2 if m["head"]["res"].get("split_variant") in (1, 2) else 1)
                             + (ph.get("gemm", {}).get("calls", 0) * 3 * (m["split"]["pipe_groups"] - 1)
                                if m["head"]["res"].get("split_variant") == 2 else 0)),
         "roofline": m["roofline"],
