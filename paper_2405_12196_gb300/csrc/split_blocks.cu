@@ -9,7 +9,9 @@
 //   split_rowmax_kernel: the item's row maxima of the biased exponent, read
 //                        straight into registers (two items per CTA), combined
 //                        over the row's items into its scale exponent with
-//                        atomicMax (and into the operand's largest);
+//                        atomicMax (and into the operand's largest); short lists
+//                        take split_rowmax_tile_kernel (one item per CTA, through
+//                        shared memory);
 //   split_digits_kernel: the whole item loaded into a shared-memory tile of raw
 //                        FP64 bits with asynchronous copies, every element in
 //                        flight at once, then the balanced digits at the row
@@ -49,6 +51,21 @@ __device__ __forceinline__ void cp_async8(void *smem_dst, const void *gsrc) {
                "l"(gsrc)
                : "memory");
 }
+
+// What a tile keeps of the double at p: all its bits (the digits kernel), or the upper
+// word (the row maxima need the exponent alone).
+__device__ __forceinline__ void fetch(unsigned long long *dst, const double *p) { cp_async8(dst, p); }
+__device__ __forceinline__ void fetch(uint32_t *dst, const double *p) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(reinterpret_cast<const uint32_t *>(p) + 1)
+               : "memory");
+}
+
+// The row-maxima kernel's shared memory: the upper words of the item (16.6 KB).
+struct __align__(16) MaxSmem {
+  uint32_t tile[kItemRows][kPitch];
+  int rmax[kItemRows];
+};
 
 // The digits kernel's shared memory: the item's tile of raw FP64 bits and its
 // rows' scale exponents (33.2 KB).
@@ -152,8 +169,8 @@ struct Walk<1> {
 // range is mostly shorter than the item's 128: one pass per 32 instead of four copies
 // per row, most of them masked off). ND: the dims of the stepped side (K when rfast,
 // else the rows).
-template <int ND>
-__device__ __forceinline__ void load_units(Smem &sm, const SliceSeg &g, int u0, int u1, int lane,
+template <int ND, class S>
+__device__ __forceinline__ void load_units(S &sm, const SliceSeg &g, int u0, int u1, int lane,
                                            const double *__restrict__ X) {
   const int r0 = g.r0, nr = g.r1 - g.r0, k0 = g.k0, kc = g.k1 - g.k0;
   const double *base = X + g.boff;
@@ -161,20 +178,20 @@ __device__ __forceinline__ void load_units(Smem &sm, const SliceSeg &g, int u0, 
   if (g.rfast) {
     if (lane < nr) {
       w.start(base + side_offset(g.ibase + lane, g.nf, g.fext, g.fst), g.kbase + u0, g.kext, g.kst);
-      unsigned long long *t = &sm.tile[r0 + lane][k0 + u0];
+      auto *t = &sm.tile[r0 + lane][k0 + u0];
 #pragma unroll 4
       for (int k = u0; k < u1; k++) {
-        cp_async8(t++, w.at());
+        fetch(t++, w.at());
         w.step();
       }
     }
   } else {
     for (int k = lane; k < kc; k += 32) {
       w.start(base + side_offset(g.kbase + k, g.nk, g.kext, g.kst), g.ibase + u0, g.fext, g.fst);
-      unsigned long long *t = &sm.tile[r0 + u0][k0 + k];
+      auto *t = &sm.tile[r0 + u0][k0 + k];
 #pragma unroll 4
       for (int r = u0; r < u1; r++) {
-        cp_async8(t, w.at());
+        fetch(t, w.at());
         t += kPitch;
         w.step();
       }
@@ -182,7 +199,8 @@ __device__ __forceinline__ void load_units(Smem &sm, const SliceSeg &g, int u0, 
   }
 }
 
-__device__ __forceinline__ void load_units_any(Smem &sm, const SliceSeg &g, int u0, int u1, int lane,
+template <class S>
+__device__ __forceinline__ void load_units_any(S &sm, const SliceSeg &g, int u0, int u1, int lane,
                                                const double *__restrict__ X) {
   switch (g.rfast ? g.nk : g.nf) {
     case 0: load_units<0>(sm, g, u0, u1, lane, X); break;
@@ -239,7 +257,8 @@ __device__ __forceinline__ void for_warp_share(const SliceItem &it, const SliceS
 
 // The item's 32 x 128 elements into the tile (zero where no block lies), offsets
 // decomposed once per lane and part and stepped after that.
-__device__ __forceinline__ void load_item(Smem &sm, const SliceItem &it, const SliceSeg *__restrict__ segs,
+template <class S>
+__device__ __forceinline__ void load_item(S &sm, const SliceItem &it, const SliceSeg *__restrict__ segs,
                                           const double *__restrict__ X) {
   const int tid = threadIdx.x, lane = tid & 31;
   if (!it.full) {   // the whole tile, pitch padding included, in 16-byte stores
@@ -263,10 +282,10 @@ __device__ __forceinline__ int biased_exp_at(const double *p) {
 // step of the lanes along K, 32 at a time, its maximum reduced over the warp, eight rows
 // in flight. A warp's part of a segment is short (some ten steps), so the last, partial
 // batch issues its loads together too, and a side merged to one dim is stepped by an
-// addition: 93 -> 89 us on the D = 12 operands (3.1e7 elements), 1283 -> 1219 us on D =
-// 20. Latency-bound all the same (loads waited for, issue slots a third busy): registers
-// for six CTAs per SM instead of eight gave 80 and 1302 us. ND: the dims of the stepped
-// side.
+// addition: 93 -> 89 us on the D = 12 operands (3.1e7 elements; 79 us now, with the tile
+// kernel), 1283 -> 1219 us on D = 20. Latency-bound all the same (loads waited for, issue
+// slots a third busy): registers for six CTAs per SM instead of eight gave 80 and 1302
+// us. ND: the dims of the stepped side.
 template <int ND>
 __device__ __forceinline__ void rowmax_units(int *rmax, const SliceSeg &g, int u0, int u1, int lane,
                                              const double *__restrict__ X) {
@@ -381,6 +400,44 @@ __global__ void __launch_bounds__(kThreads, 8) split_rowmax_kernel(const SplitOp
   }
 }
 
+// The same maxima, one item per CTA, through a shared-memory tile of the elements' upper
+// words: every element in flight at once, none of them held in a register, then each row
+// read back by one warp. For short lists of items (kRowmaxTileItems).
+__global__ void __launch_bounds__(kThreads, 8) split_rowmax_tile_kernel(const SplitOperand *__restrict__ ops,
+                                                                        const SliceItem *__restrict__ items,
+                                                                        const SliceSeg *__restrict__ segs,
+                                                                        const double *__restrict__ a,
+                                                                        const double *__restrict__ b,
+                                                                        int32_t *__restrict__ ea,
+                                                                        int32_t *__restrict__ eb,
+                                                                        int32_t *__restrict__ emax) {
+  __shared__ MaxSmem sm;
+  after_previous_kernel();
+  const SliceItem it = items[blockIdx.x];
+  const bool isA = (it.op & 1) == 0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nq = min(kItemK / 32, ops[it.op].ks - it.kq * (kItemK / kSplitBK));   // K stages the operand has here
+  load_item(sm, it, segs, isA ? a : b);
+#pragma unroll
+  for (int rr = warp; rr < kItemRows; rr += kThreads / 32) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int q = 0; q < kItemK / 32; q++)
+      if (q < nq) m = max(m, sm.tile[rr][q * 32 + lane] & 0x7FF00000u);   // the rest is not written
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) sm.rmax[rr] = (int)(m >> 20);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const SplitOperand &o = ops[it.op];
+    const int row = it.rt * kSplitBM + it.quarter * kItemRows + lane;
+    const int m = row < o.rows ? sm.rmax[lane] : 0;
+    if (row < o.rows) atomicMax((isA ? ea : eb) + o.exp_off + row, m);
+    const int all = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) atomicMax(emax + it.op, all);
+  }
+}
+
 // MINB: CTAs per SM the launch bounds ask for. 5: 48 registers (five CTAs per SM,
 // as shared memory allows), the fastest alone; 6: 40
 // registers, so that one CTA fits beside a split-GEMM CTA of four slices (576 threads x
@@ -430,6 +487,15 @@ cudaError_t configure_split_blocks() {
                               cudaSharedmemCarveoutMaxShared);
 }
 
+// Lists of fewer items take the tile kernel: about ten waves of eight CTAs on each of 152
+// SMs. With few waves its finer grain and its loads without a wait between them are
+// faster: D = 10 run (4288 items) 38.9 -> 37.0 us, D = 12 environment (9408) 89 -> 79 us,
+// complex D = 8 run (1560) 131 -> 126 us for the whole contraction. On long lists the two
+// items per CTA of the other kernel hide more of the tables' latency: D = 13 (16,936) 1168
+// against 1175 us for the whole contraction, D = 16 (34,104) 2413 against 2427, D = 20
+// (176,328) 1219 against 1391 us for the kernel.
+constexpr int64_t kRowmaxTileItems = 12000;
+
 cudaError_t launch_split_blocks(const SplitOperand *ops, const SliceItem *items, int64_t nitems,
                                 const SliceSeg *segs, const double *a, const double *b, int32_t *ea, int32_t *eb,
                                 int32_t *emax, uint8_t *sa, uint8_t *sb, int slices, bool beside_gemm,
@@ -437,8 +503,13 @@ cudaError_t launch_split_blocks(const SplitOperand *ops, const SliceItem *items,
   if (nitems <= 0) return cudaSuccess;
   if (nitems > INT32_MAX || slices < 1 || slices > kSlices) return cudaErrorInvalidValue;
   const unsigned g0 = (unsigned)((nitems + kRowmaxItems - 1) / kRowmaxItems);
-  cudaError_t e = launch_chained(beside_gemm ? split_rowmax_kernel<true> : split_rowmax_kernel<false>, g0, kThreads, 0,
-                                 stream, ops, items, (int)nitems, segs, a, b, ea, eb, emax);
+  cudaError_t e;
+  if (!beside_gemm && nitems < kRowmaxTileItems)
+    e = launch_chained(split_rowmax_tile_kernel, (unsigned)nitems, kThreads, 0, stream, ops, items, segs, a, b, ea, eb,
+                       emax);
+  else
+    e = launch_chained(beside_gemm ? split_rowmax_kernel<true> : split_rowmax_kernel<false>, g0, kThreads, 0, stream,
+                       ops, items, (int)nitems, segs, a, b, ea, eb, emax);
   if (e == cudaSuccess)
     e = launch_chained(beside_gemm ? split_digits_kernel<6> : split_digits_kernel<5>, (unsigned)nitems, kThreads, 0, stream,
                        ops, items, segs, a, b, ea, eb, sa, sb, slices);
