@@ -55,7 +55,7 @@
 // 1.86e12 FLOPs) a stage took 2940 clocks with one CTA per 128 x 128 tile (18.1 ms, and
 // 0.9 ms for the scatter of C) and takes 2180 (15.6 ms with C written, at 1.77 instead
 // of 1.95 GHz: the power limit now takes part of the gain); D = 12 (30 GFLOP): 416 + 45
-// us -> 350 us.
+// us -> 320 us.
 // Every wait is bounded; on expiry the kernel records a status code, stops
 // issuing work, waits (bounded) for its own copies and MMAs and frees tensor
 // memory before returning.
