@@ -57,8 +57,8 @@
 // of 1.95 GHz: the power limit now takes part of the gain); D = 12 (30 GFLOP): 416 + 45
 // us -> 320 us.
 // Every wait is bounded; on expiry the kernel records a status code, stops
-// issuing work, waits (bounded) for its own copies and MMAs and frees tensor
-// memory before returning.
+// issuing work, waits (bounded, whatever the abort flag says: mbar_drain) for its own
+// copies and MMAs and frees tensor memory before returning.
 #include <cuda_runtime.h>
 
 #include "kernels.hpp"
@@ -73,6 +73,7 @@ constexpr int kEpiWarps = 16;
 constexpr int kHalfBytes = kSliceBytes / 2;   // a CTA's half of a Q slice
 constexpr uint32_t kColE2 = 0, kColE3 = 128, kColE4 = 256, kColR = 384;
 constexpr uint32_t kMaxPolls = 1u << 26;
+constexpr uint32_t kDrainPolls = 1u << 18;
 constexpr int kOutGroup = 8;    // rows of Q converted without a look at C's blocks in between
 constexpr int kMaxStarts = 4;   // blocks of C among a warp's 32 rows with places read ahead
 
@@ -182,6 +183,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   abort_pair(abort_flag);
   atomicCAS(status, 0, code);
   return false;
+}
+
+// A last look at a phase that mbar_wait gave up on: the bulk copies and MMAs already issued
+// go on after an abort, and a CTA keeps its shared and tensor memory until they have
+// ended. They end within microseconds; kDrainPolls tests take a few milliseconds (a slot
+// of the leader whose peer stopped before its copy never completes: then the bound ends it).
+__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
+  for (uint32_t i = 0; i < kDrainPolls && !mbar_test(bar, parity); i++) {}
 }
 
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
@@ -505,7 +514,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     // ---------------------------------------------------------------- producer
     if (lane == 0) {
       Slot lead, rest;
-      uint32_t loads = 0;
+      uint32_t nlead = 0, nrest = 0;   // slots loaded
       bool ok = true;
       for (int t = pair; t < ntiles && ok; t += npairs) {
         const SplitTile tl = tiles[t];
@@ -531,25 +540,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
               bulk_g2s(dst + pbytes + p * qbytes, qblk + (p0 + p) * kSliceBytes, qbytes, fb);
           };
           load(kFull0, kEmpty0, lead, smem_u32(smem) + lead.i * RG::kLeadSlot, 0, 3);
-          if (ok)
-            load(kRestFull0, kRestEmpty0, rest, smem_u32(smem) + RG::kLeadBytes + rest.i * RG::kRestSlot, 3, RG::kRest);
           if (!ok) break;
-          loads++;
+          nlead++;
           lead.next(RG::kLeadStages);
+          load(kRestFull0, kRestEmpty0, rest, smem_u32(smem) + RG::kLeadBytes + rest.i * RG::kRestSlot, 3, RG::kRest);
+          if (!ok) break;
+          nrest++;
           rest.next(RG::kRestStages);
         }
       }
       // no copy, and no arrival of a "slot free" commit, may still be in flight when
-      // the CTA exits
-      for (uint32_t k = 1; k <= (uint32_t)RG::kLeadStages && k <= loads; k++) {
-        lead.back(RG::kLeadStages);
-        mbar_wait(bar(kFull0 + lead.i), lead.phase, abort_flag, status, 2);
-        mbar_wait(bar(kEmpty0 + lead.i), lead.phase, abort_flag, status, 10);
-        if (k > (uint32_t)RG::kRestStages) continue;
-        rest.back(RG::kRestStages);
-        mbar_wait(bar(kRestFull0 + rest.i), rest.phase, abort_flag, status, 2);
-        mbar_wait(bar(kRestEmpty0 + rest.i), rest.phase, abort_flag, status, 10);
-      }
+      // the CTA exits (after an abort some slots are never freed: those waits end with
+      // the flag, and the commits that were issued are waited for through kDone)
+      auto finish = [&](Slot &sl, uint32_t n, int stages, int full, int empty) {
+        for (uint32_t k = 0; k < min(n, (uint32_t)stages); k++) {
+          sl.back(stages);
+          if (!mbar_wait(bar(full + sl.i), sl.phase, abort_flag, status, 2)) mbar_drain(bar(full + sl.i), sl.phase);
+          mbar_wait(bar(empty + sl.i), sl.phase, abort_flag, status, 10);
+        }
+      };
+      finish(lead, nlead, RG::kLeadStages, kFull0, kEmpty0);
+      finish(rest, nrest, RG::kRestStages, kRestFull0, kRestEmpty0);
     }
   } else if (warp == 1 && rank == 1) {
     // --------------------------------------------------------- relay (peer CTA)
@@ -569,6 +580,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           rest.next(RG::kRestStages);
         }
       }
+      // the leader's MMAs read this CTA's shared memory and their commits arrive here
+      if (!mbar_wait(bar(kDone), 0, abort_flag, status, 6)) mbar_drain(bar(kDone), 0);
     }
   } else if (warp == 1) {
     // --------------------------------------------------------- MMA issuer (leader)
@@ -666,11 +679,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
     // every issued MMA has completed before tensor memory is released
     __syncwarp();
-    if (elect_one())
-      asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar(kDone))
-                   : "memory");
+    if (elect_one()) umma_commit(bar(kDone));
     __syncwarp();
-    if (lane == 0) mbar_wait(bar(kDone), 0, abort_flag, status, 6);
+    if (lane == 0 && !mbar_wait(bar(kDone), 0, abort_flag, status, 6)) mbar_drain(bar(kDone), 0);
   } else if (warp >= kFirstEpiWarp) {
     // ---------------------------------------------------------------- epilogue
     // four warps per 32-lane quarter of tensor memory; columns [c0, c0 + w) with
