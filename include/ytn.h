@@ -381,7 +381,8 @@ ytn_status ytn_workspace_size_staged(const ytn_plan_t *plan, ytn_precision prec,
  * cudaHostRegister, mapped into the device's address space). Host-resident
  * data is read (and C written) by the data-mover kernels directly over the
  * host link, with no staging copy. Pageable host memory is rejected
- * (YTN_E_INVALID). Every element of c is written. prec/rtol select the product precision (rtol is the target
+ * (YTN_E_INVALID). Every element of c is written. c may overlap a or b, which it then
+ * overwrites (at the price of a second pass over C). prec/rtol select the product precision (rtol is the target
  * relative Frobenius error of the split path, ignored for FP64).
  * workspace: device buffer of at least ytn_workspace_size bytes, 256-byte
  * aligned. res (optional, host): filled before return. Asynchronous on stream.
@@ -390,7 +391,8 @@ ytn_status ytn_workspace_size_staged(const ytn_plan_t *plan, ytn_precision prec,
  * the first such call times both paths on the caller's stream (it runs both,
  * leaves the split result in c and synchronises the stream); later calls reuse
  * the cached choice. While the stream is being captured into a graph, a cost
- * model of the two kernels' tile-padded work decides instead. res->precision
+ * model of the two kernels' tile-padded work decides instead, and likewise (for that
+ * call alone, for every choice named here) where c overlaps a or b. res->precision
  * reports the path that wrote c; the workspace is ytn_workspace_size(YTN_AUTO).
  * The split path has two variants for plans whose blocks have at most three
  * dims per side (ytn_plan_info.split_fused): slices built straight from the

@@ -975,7 +975,8 @@ ytn_status ytn_tensordot(ytn_plan_t *p, const double *a, const double *b, double
     const char *p0 = reinterpret_cast<const char *>(x), *c0 = reinterpret_cast<const char *>(c);
     return p0 + n <= c0 || c0 + bytes_c <= p0;
   };
-  const bool direct = (!hc || staged) && apart(a, bytes_a) && apart(b, bytes_b);
+  const bool overlap = !apart(a, bytes_a) || !apart(b, bytes_b);
+  const bool direct = (!hc || staged) && !overlap;
   auto unstage = [&]() -> ytn_status {
     if (!staged || !hc || !p->out.size) return YTN_OK;
     const size_t wc = (size_t)p->out.size * (p->out.dtype == YTN_COMPLEX128 ? 16 : 8);
@@ -999,7 +1000,9 @@ ytn_status ytn_tensordot(ytn_plan_t *p, const double *a, const double *b, double
   // list (all 128 wide, or with 64-wide sector tails when the plan has any). The
   // first call that needs a choice times the candidates on the caller's stream
   // (this call synchronises it; C holds the last candidate's result, a split
-  // result); under graph capture cost models decide.
+  // result); under graph capture cost models decide. So they do where C overlaps an
+  // operand, which the first candidate would overwrite for the next: for this call
+  // alone, a later one with C apart from the operands still times the candidates.
   int choice = 1, variant = 0, tiles = 0;
   if (prec == YTN_AUTO) {
     if (!split_ok) {
@@ -1019,14 +1022,15 @@ ytn_status ytn_tensordot(ytn_plan_t *p, const double *a, const double *b, double
   const bool need_choice = prec == YTN_AUTO && split_ok && choice < 0;
   const bool need_variant = may_split && p->sp_fused && variant < 0;
   const bool need_tiles = may_split && has_mix && tiles < 0;
-  if ((need_choice || need_variant || need_tiles) && capturing) {
+  if ((need_choice || need_variant || need_tiles) && (capturing || overlap)) {
     std::lock_guard<std::mutex> lk(p->auto_mu);
-    if (need_choice && p->auto_choice[slices] < 0) p->auto_choice[slices] = model_prefers_split(p, slices) ? 1 : 0;
-    if (p->sp_fused && p->split_variant[slices] < 0) p->split_variant[slices] = model_prefers_fused(p) ? 1 : 0;
-    if (has_mix && p->tile_policy[slices] < 0) p->tile_policy[slices] = 0;
-    choice = prec == YTN_AUTO ? p->auto_choice[slices] : 1;
-    variant = p->sp_fused ? p->split_variant[slices] : 0;
-    tiles = has_mix ? p->tile_policy[slices] : 0;
+    auto decide = [&](int &kept, int model) {
+      if (kept < 0 && capturing) kept = model;
+      return kept < 0 ? model : kept;
+    };
+    if (need_choice) choice = decide(p->auto_choice[slices], model_prefers_split(p, slices) ? 1 : 0);
+    if (p->sp_fused) variant = decide(p->split_variant[slices], model_prefers_fused(p) ? 1 : 0);
+    if (has_mix) tiles = decide(p->tile_policy[slices], 0);
   } else if (need_choice || need_variant || need_tiles) {
     // candidates in a fixed order: FP64 (YTN_AUTO), staged split, fused split (128
     // wide tiles), then the variant of the previous run with 64-wide tails
