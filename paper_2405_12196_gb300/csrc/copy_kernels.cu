@@ -355,6 +355,13 @@ __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const TraceChunk *
   if (worker == 0 && lane < ne) dst[o.dst_off + ch.e0 + lane] = part[lane];
 }
 
+// x with -0 as +0, as a sum that starts from +0 gives it (an FP64 addition more per element
+// cost 1 us of the 10 of the D = 8 run's scatter).
+__device__ __forceinline__ double plus_zero(double x) {
+  const long long b = __double_as_longlong(x);
+  return __longlong_as_double(b == (long long)kSignBit ? 0ll : b);
+}
+
 // Scatter-combine of a complex product: the doubled real C_q holds the four
 // real products in quadrants; a CTA writes kCScatterElems elements of one C block,
 // re = P00 - P11 and im = P01 + P10 (absent quadrants, from a real operand, count as
@@ -388,7 +395,7 @@ __global__ void __launch_bounds__(256) cscatter_kernel(const CScatterJob *__rest
 #pragma unroll
   for (int u = 0; u < kPer; u++) {
     const uint32_t e = (uint32_t)ch.e0 + threadIdx.x + 256 * u;
-    if (e < (uint32_t)J.n) out[e] = make_double2(r0[u] - r1[u], i0[u] + i1[u]);
+    if (e < (uint32_t)J.n) out[e] = make_double2(r0[u] - r1[u], plus_zero(i0[u] + i1[u]));
   }
 }
 

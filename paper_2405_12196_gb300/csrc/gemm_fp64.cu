@@ -225,7 +225,7 @@ __device__ __forceinline__ void outer_tile(const SectorDev &s, const GemmTile &t
       blk = row.blk;
       base = __ldg(out.base + so.base + (int64_t)blk * so.ncb + col.blk);
     }
-    double v = As[0][r] * b[0];
+    double v = fma(As[0][r], b[0], 0.0);   // a sum from +0, as the DMMA steps': no -0 from a zero factor
     if (K > 1) v = fma(As[1][r], b[1], v);
     if (base >= 0) out.c[base + (int64_t)row.idx * col.len + col.idx] = v;
   }
