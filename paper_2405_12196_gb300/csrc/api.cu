@@ -82,6 +82,8 @@ static ytn_status upload(ytn_plan_t *p) {
   put_table(buf, p->sp_exp_items, o_spe);
   put_table(buf, p->sp_slice_items, o_sps);
   put_table(buf, p->sp_sectors, o_spsec);
+  size_t o_spck;
+  put_table(buf, p->sp_checks, o_spck);
   put_table(buf, p->sp_tiles, o_spt);
   size_t o_sptm;
   put_table(buf, p->sp_tiles_mix, o_sptm);
@@ -120,6 +122,7 @@ static ytn_status upload(ytn_plan_t *p) {
   p->d_sp_exp_items = reinterpret_cast<const SplitItem *>(d + o_spe);
   p->d_sp_slice_items = reinterpret_cast<const SplitItem *>(d + o_sps);
   p->d_sp_sectors = reinterpret_cast<const SplitSector *>(d + o_spsec);
+  p->d_sp_checks = reinterpret_cast<const SplitCheckChunk *>(d + o_spck);
   p->d_sp_tiles = reinterpret_cast<const SplitTile *>(d + o_spt);
   p->d_sp_tiles_pipe = reinterpret_cast<const SplitTile *>(d + o_sptp);
   p->d_sp_tiles_mix = reinterpret_cast<const SplitTile *>(d + o_sptm);
@@ -217,10 +220,10 @@ static void note_capture(ytn_plan_t *p, cudaStream_t st) {
 // SA | SB (BF16 slice blocks) | EA | EB (row / column exponents) and the accuracy
 // check: EMAX | NORMSQ | REC | SECV | FLAGGED | TILE_END (see SplitRecord);
 // 256-byte aligned regions, except that EMAX follows EB directly; one memset covers EA to
-// SECV.
+// REC.
 struct WsLayout {
   size_t wa = 0, wb = 0, wc = 0, sa = 0, sb = 0, ea = 0, eb = 0;
-  size_t emax = 0, normsq = 0, rec = 0, rec_end = 0, secv = 0, secv_end = 0, flagged = 0, tile_end = 0;
+  size_t emax = 0, normsq = 0, rec = 0, rec_end = 0, secv = 0, flagged = 0, tile_end = 0;
   size_t item_end_a = 0, item_end_b = 0;
 };
 
@@ -252,8 +255,7 @@ static size_t workspace_layout(const ytn_plan_t *p, bool split, WsLayout &w) {
   w.rec_end = o;
   o = align256(o);
   w.secv = o;
-  o += align256(nsec * 16);
-  w.secv_end = o;
+  o += align256(p->sp_checks.size() * 16);
   w.flagged = o;
   o += align256(nsec * 4);
   w.tile_end = o;
@@ -796,7 +798,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
       if (e == cudaSuccess) e = cudaStreamWaitEvent(hi, ev(0), 0);
       if (e == cudaSuccess) {
         PhaseTimer t(p->ctx, YTN_PHASE_SPLIT, hi);
-        e = cudaMemsetAsync(ea, 0, w.secv_end - w.ea, hi);
+        e = cudaMemsetAsync(ea, 0, w.rec_end - w.ea, hi);
         if (e == cudaSuccess)
           e = launch_split_blocks(p->d_sp_ops, p->d_sp_fitems, ie[0], p->d_sp_segs, a, b, ea, eb, emax, sa, sb, slices,
                                   false, hi);
@@ -828,8 +830,8 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
       {
         PhaseTimer t(p->ctx, YTN_PHASE_SPLIT, st);
         // the exponent kernels max-combine into EA, EB and EMAX, the epilogue sums into
-        // NORMSQ, the check into SECV and counts in the record: all start from zero
-        e = cudaMemsetAsync(ea, 0, w.secv_end - w.ea, st);
+        // NORMSQ and the check counts in the record: all start from zero
+        e = cudaMemsetAsync(ea, 0, w.rec_end - w.ea, st);
         if (e == cudaSuccess) {
           if (fused)
             e = launch_split_blocks(p->d_sp_ops, p->d_sp_fitems, (int64_t)p->sp_fitems.size(), p->d_sp_segs, a, b,
@@ -857,7 +859,8 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
       int32_t *tile_end = reinterpret_cast<int32_t *>(ws + w.tile_end);
       int32_t *item_end_a = reinterpret_cast<int32_t *>(ws + w.item_end_a);
       int32_t *item_end_b = reinterpret_cast<int32_t *>(ws + w.item_end_b);
-      e = launch_split_check(p->d_sp_sectors, (int64_t)p->sp_sectors.size(), p->max_m + p->max_n, ea, eb, emax, normsq,
+      e = launch_split_check(p->d_sp_sectors, (int64_t)p->sp_sectors.size(), p->d_sp_checks,
+                             (int64_t)p->sp_checks.size(), ea, eb, emax, normsq,
                              reinterpret_cast<double *>(ws + w.secv), flagged, tile_end, item_end_a, item_end_b, rec,
                              split_eta(slices), kEtaFp64, rtol, slices, p->ctx->status_dev, st);
       if (e == cudaSuccess && fused && !p->sp_sectors.empty())

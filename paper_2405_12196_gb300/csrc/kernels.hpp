@@ -103,13 +103,12 @@ cudaError_t launch_gemm_split(const SplitSector *sectors, const SplitTile *tiles
 // sectors above rtol with their 64 x 64 tile counts, the call's record, and the
 // status word's tolerance flag (status[1]) when the fallback cannot reach rtol.
 // eta_split / eta_fp64: per-element error of the split / FP64 products relative
-// to the row and column scales, per square root of K. max_rows: the largest M + N of a
-// sector; secv: two zeros per sector.
-cudaError_t launch_split_check(const SplitSector *sectors, int64_t nsec, int64_t max_rows, const int32_t *ea,
-                               const int32_t *eb, const int32_t *emax, const float *normsq, double *secv,
-                               int32_t *flagged, int32_t *tile_end, int32_t *item_end_a, int32_t *item_end_b,
-                               SplitRecord *rec, double eta_split, double eta_fp64, double rtol, int slices,
-                               int *status, cudaStream_t stream);
+// to the row and column scales, per square root of K. secv: two values per chunk.
+cudaError_t launch_split_check(const SplitSector *sectors, int64_t nsec, const SplitCheckChunk *chunks,
+                               int64_t nchunks, const int32_t *ea, const int32_t *eb, const int32_t *emax,
+                               const float *normsq, double *secv, int32_t *flagged, int32_t *tile_end,
+                               int32_t *item_end_a, int32_t *item_end_b, SplitRecord *rec, double eta_split,
+                               double eta_fp64, double rtol, int slices, int *status, cudaStream_t stream);
 
 // FP64 fallback of the fused split path: zero fill (partially populated
 // operands) and gathers of the flagged sectors' FP64 sector matrices only

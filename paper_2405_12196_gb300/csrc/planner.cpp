@@ -1278,6 +1278,7 @@ void plan_split_tables(ytn_plan_t *p, std::vector<SegSource> *src) {
   p->sp_exp_items.clear();
   p->sp_slice_items.clear();
   p->sp_sectors.clear();
+  p->sp_checks.clear();
   p->sp_tiles.clear();
   p->sp_tiles_mix.clear();
   p->sp_fitems.clear();
@@ -1306,6 +1307,10 @@ void plan_split_tables(ytn_plan_t *p, std::vector<SegSource> *src) {
       s.gb0 = (int32_t)p->sec_gather_items[q][2];
       s.gb1 = (int32_t)p->sec_gather_items[q][3];
     }
+    s.chk0 = (int32_t)p->sp_checks.size();
+    const int64_t nchk = ((h.M + 3) / 4 * 4 + h.N + kCheckRows - 1) / kCheckRows;
+    for (int64_t i = 0; i < nchk; i++) p->sp_checks.push_back({(int32_t)q, (int32_t)i});
+    s.chk1 = (int32_t)p->sp_checks.size();
     p->sp_sectors.push_back(s);
     SplitOperand oa{h.a_off, ea, sa, (int32_t)h.M, (int32_t)h.K, (int32_t)ks, p->a_kmajor ? 1 : 0};
     SplitOperand ob{h.b_off, eb, sb, (int32_t)h.N, (int32_t)h.K, (int32_t)ks, p->b_kmajor ? 1 : 0};

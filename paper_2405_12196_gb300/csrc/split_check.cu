@@ -12,10 +12,11 @@
 // large element and the rest far below it, or when the products cancel, the
 // scales are large against |c_ij| and the estimate grows with that ratio.
 //
-// A CTA sums the scales of kRows rows of one sector's operands (both taken relative
+// A CTA sums the scales of kCheckRows rows of one sector's operands (both taken relative
 // to the operands' largest exponents, so nothing overflows): FP64 additions are slow on
 // this GPU, two a clock and SM, so the rows of a large sector are shared out (one CTA
-// per sector took 83 us for two sectors of 133,000 rows and columns). The last CTA to
+// per sector took 83 us for two sectors of 133,000 rows and columns). The sums are added
+// in a fixed order, within a CTA and over a sector's CTAs. The last CTA to
 // finish, from these and the ||C_q||^2 that the GEMM epilogue summed, with one division
 // per sector and the lists only when a sector is flagged (a chain of latencies: square
 // roots and four prefix sums per sector made it 17 to 24 us, now 13 to 14):
@@ -42,7 +43,7 @@ namespace ytn {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kRows = 4096;   // rows of A and B together that one CTA sums
+constexpr int kFewChunks = 4;   // a sector's chunks that one thread adds
 
 // 4^k for k <= 0 as an FP64 value built from its bits (0 below the normal range).
 __device__ __forceinline__ double pow4(int k) {
@@ -56,9 +57,9 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // This thread's share of the sum of 4^(e[i] - E) over rows [lo, hi).
-__device__ __forceinline__ double scale_sum(const int32_t *__restrict__ e, int lo, int hi, int E) {
+__device__ __forceinline__ double scale_sum(const int32_t *__restrict__ e, uint32_t lo, uint32_t hi, int E) {
   double s = 0.0;
-  int i = lo + 4 * (int)threadIdx.x;
+  uint32_t i = lo + 4 * threadIdx.x;
 #pragma unroll 4
   for (; i + 4 <= hi; i += 4 * kThreads) {   // rows start on multiples of 128
     const int4 x = *reinterpret_cast<const int4 *>(e + i);
@@ -92,7 +93,8 @@ __device__ __forceinline__ int block_scan(int v, int *red, int *total) {
 }
 
 __global__ void __launch_bounds__(kThreads) split_check_kernel(
-    const SplitSector *__restrict__ sectors, int nsec, int nchunk, const int32_t *__restrict__ ea,
+    const SplitSector *__restrict__ sectors, int nsec, const SplitCheckChunk *__restrict__ chunks,
+    const int32_t *__restrict__ ea,
     const int32_t *__restrict__ eb, const int32_t *__restrict__ emax, const float *__restrict__ normsq, double *secv,
     int32_t *__restrict__ flagged, int32_t *__restrict__ tile_end, int32_t *__restrict__ item_end_a,
     int32_t *__restrict__ item_end_b, SplitRecord *rec, double eta_split, double eta_fp64, double rtol, int slices,
@@ -101,20 +103,31 @@ __global__ void __launch_bounds__(kThreads) split_check_kernel(
   __shared__ int ired[kThreads / 32];
   __shared__ int is_last;
   after_previous_kernel();
-  const int q = blockIdx.x / nchunk, chunk = blockIdx.x - q * nchunk, tid = threadIdx.x;
+  // a chunk per sector: the tables need no look (0.5 us on the D = 10 run)
+  const bool single = nsec == (int)gridDim.x;
+  const SplitCheckChunk ch = single ? SplitCheckChunk{(int)blockIdx.x, 0} : chunks[blockIdx.x];
+  const int q = ch.sector, tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
   {
     const SplitSector sc = sectors[q];
-    const int lo = chunk * kRows, hi = lo + kRows;   // rows of A, then of B from align4(M) on
-    const int mb = (sc.M + 3) & ~3;
+    // rows of A, then of B from align4(M) on
+    const int64_t lo = (int64_t)ch.idx * kCheckRows, hi = lo + kCheckRows, mb = ((int64_t)sc.M + 3) & ~(int64_t)3;
     double se = 0.0, sf = 0.0;
-    if (lo < sc.M) se = scale_sum(ea + sc.ea_off, lo, min(sc.M, hi), emax[2 * q]);
-    if (hi > mb && lo - mb < sc.N) sf = scale_sum(eb + sc.eb_off, max(0, lo - mb), min(sc.N, hi - mb), emax[2 * q + 1]);
+    if (lo < sc.M) se = scale_sum(ea + sc.ea_off, lo, min((int64_t)sc.M, hi), emax[2 * q]);
+    if (hi > mb && lo - mb < sc.N)
+      sf = scale_sum(eb + sc.eb_off, max((int64_t)0, lo - mb), min((int64_t)sc.N, hi - mb), emax[2 * q + 1]);
     se = warp_sum(se);
     sf = warp_sum(sf);
     if (lane == 0) {
-      if (se > 0.0) atomicAdd(secv + 2 * q, se);
-      if (sf > 0.0) atomicAdd(secv + 2 * q + 1, sf);
+      dred[0][warp] = se;
+      dred[1][warp] = sf;
+    }
+    __syncthreads();
+    if (tid < 2) {
+      double t = 0.0;
+#pragma unroll
+      for (int w = 0; w < kThreads / 32; w++) t += dred[tid][w];
+      secv[2 * blockIdx.x + tid] = t;
     }
   }
   // the last CTA to get here sees every sector's sums
@@ -125,10 +138,46 @@ __global__ void __launch_bounds__(kThreads) split_check_kernel(
   if (!is_last) return;
   __threadfence();
 
+  // the sums of sectors of several chunks into their first chunk's place, by the thread that
+  // looks at the sector below (of more than kFewChunks: its warp)
+  for (int base = 0; base < nsec && !single; base += kThreads) {
+    const int s = base + tid;
+    int c0 = 0, n = 0;
+    if (s < nsec) {
+      c0 = sectors[s].chk0;
+      n = sectors[s].chk1 - c0;
+    }
+    double se = 0.0, sf = 0.0;
+    if (n > 1 && n <= kFewChunks)
+      for (int c = c0; c < c0 + n; c++) {
+        se += __ldcg(secv + 2 * c);
+        sf += __ldcg(secv + 2 * c + 1);
+      }
+    for (uint32_t many = __ballot_sync(0xffffffffu, n > kFewChunks); many; many &= many - 1) {
+      const int b = __ffs(many) - 1;
+      const int from = __shfl_sync(0xffffffffu, c0, b), to = from + __shfl_sync(0xffffffffu, n, b);
+      double pe = 0.0, pf = 0.0;
+      for (int c = from + lane; c < to; c += 32) {
+        pe += __ldcg(secv + 2 * c);
+        pf += __ldcg(secv + 2 * c + 1);
+      }
+      pe = warp_sum(pe);
+      pf = warp_sum(pf);
+      if (lane == b) {
+        se = pe;
+        sf = pf;
+      }
+    }
+    if (n > 1) {
+      __stcg(secv + 2 * c0, se);
+      __stcg(secv + 2 * c0 + 1, sf);
+    }
+  }
   // K_q sum_i 4^(e_i - emax_A) sum_j 4^(f_j - emax_B): 0 for a zero operand
   auto value = [&](int s) {
     if (emax[2 * s] <= 0 || emax[2 * s + 1] <= 0) return 0.0;
-    return (double)sectors[s].K * __ldcg(secv + 2 * s) * __ldcg(secv + 2 * s + 1);
+    const double *v = secv + 2 * (single ? s : sectors[s].chk0);
+    return (double)sectors[s].K * __ldcg(v) * __ldcg(v + 1);
   };
   // reference exponent: the largest emax_A + emax_B among sectors with data
   int g = INT_MIN;
@@ -222,17 +271,16 @@ __global__ void __launch_bounds__(kThreads) split_check_kernel(
 
 }  // namespace
 
-cudaError_t launch_split_check(const SplitSector *sectors, int64_t nsec, int64_t max_rows, const int32_t *ea,
-                               const int32_t *eb, const int32_t *emax, const float *normsq, double *secv,
-                               int32_t *flagged, int32_t *tile_end, int32_t *item_end_a, int32_t *item_end_b,
-                               SplitRecord *rec, double eta_split, double eta_fp64, double rtol, int slices,
-                               int *status, cudaStream_t stream) {
+cudaError_t launch_split_check(const SplitSector *sectors, int64_t nsec, const SplitCheckChunk *chunks,
+                               int64_t nchunks, const int32_t *ea, const int32_t *eb, const int32_t *emax,
+                               const float *normsq, double *secv, int32_t *flagged, int32_t *tile_end,
+                               int32_t *item_end_a, int32_t *item_end_b, SplitRecord *rec, double eta_split,
+                               double eta_fp64, double rtol, int slices, int *status, cudaStream_t stream) {
   if (nsec <= 0) return cudaSuccess;
-  const int64_t nchunk = std::max<int64_t>(1, (max_rows + 4 + kRows - 1) / kRows);
-  if (nsec * nchunk > INT32_MAX) return cudaErrorInvalidValue;
-  return launch_chained(split_check_kernel, (unsigned)(nsec * nchunk), kThreads, 0, stream, sectors, (int)nsec, (int)nchunk,
-                        ea, eb, emax, normsq, secv, flagged, tile_end, item_end_a, item_end_b, rec, eta_split, eta_fp64,
-                        rtol, slices, status);
+  if (nchunks < nsec || nchunks > INT32_MAX) return cudaErrorInvalidValue;
+  return launch_chained(split_check_kernel, (unsigned)nchunks, kThreads, 0, stream, sectors, (int)nsec, chunks, ea, eb,
+                        emax, normsq, secv, flagged, tile_end, item_end_a, item_end_b, rec, eta_split, eta_fp64, rtol,
+                        slices, status);
 }
 
 }  // namespace ytn

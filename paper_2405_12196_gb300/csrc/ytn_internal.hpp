@@ -227,8 +227,16 @@ struct SplitSector {
   int64_t c_off;             // element offset of C_q in the FP64 workspace
   int32_t M, N, K, ks;
   int32_t ga0, ga1, gb0, gb1; // the sector's gather items of A and B (FP64 fallback)
+  int32_t chk0, chk1;        // the sector's chunks of the accuracy check
 };
-static_assert(sizeof(SplitSector) == 72, "SplitSector layout");
+static_assert(sizeof(SplitSector) == 80, "SplitSector layout");
+
+// A CTA's share of the accuracy check: kCheckRows rows of a sector's operands from row idx
+// kCheckRows on, A's first, then B's from align4(M) on.
+constexpr int kCheckRows = 4096;
+struct SplitCheckChunk {
+  int32_t sector, idx;
+};
 
 // One output tile of the split GEMM, computed by a pair of CTAs: 256 rows of the P
 // operand (128-row tiles 2 pt and 2 pt + 1, one per CTA) times bn rows of the Q operand
@@ -254,10 +262,12 @@ static_assert(sizeof(SplitTile) == 88, "SplitTile layout");
 //   normsq  float [nsec]      ||C_q||_F^2 times 4^-(emax_A + emax_B), summed by the
 //                             GEMM epilogue
 //   SplitRecord               the call's totals (below)
-//   secv    double [2 * nsec] sum_i 4^(e_i - emax_A) and sum_j 4^(f_j - emax_B)
+//   secv    double [2 * chunks] sum_i 4^(e_i - emax_A) and sum_j 4^(f_j - emax_B) over
+//                             each chunk's rows (SplitCheckChunk)
 //   flagged int32 [nsec]      sectors recomputed on the FP64 path, in sector order
 //   tile_end int32 [nsec]     running count of their 64 x 64 FP64 tiles
-// All of them, and the exponents before them, are zeroed before the call's kernels run.
+// EMAX to the record, and the exponents before them, are zeroed before the call's kernels
+// run; the rest is written before it is read.
 struct SplitRecord {
   double err_est;          // relative Frobenius error of C after the FP64 fallback
   double split_err_est;    // the same for the split products alone (no fallback)
@@ -487,6 +497,7 @@ struct ytn_plan_s {
   std::vector<int64_t> sp_pipe_tile_end, sp_pipe_item_end;
   std::vector<std::array<int64_t, 4>> sec_gather_items;   // per sector: A items, B items (relative)
   std::vector<ytn::SplitSector> sp_sectors;
+  std::vector<ytn::SplitCheckChunk> sp_checks;
   std::vector<ytn::SplitTile> sp_tiles, sp_tiles_pipe;   // the second in sector order, for runs of sectors
   std::vector<ytn::SplitTile> sp_tiles_mix;    // with 64-wide sector tails (empty: none)
   int64_t sp_sa_bytes = 0, sp_sb_bytes = 0, sp_ea = 0, sp_eb = 0;
@@ -508,6 +519,7 @@ struct ytn_plan_s {
   const ytn::SplitOperand *d_sp_ops = nullptr;
   const ytn::SplitItem *d_sp_exp_items = nullptr, *d_sp_slice_items = nullptr;
   const ytn::SplitSector *d_sp_sectors = nullptr;
+  const ytn::SplitCheckChunk *d_sp_checks = nullptr;
   const ytn::SplitTile *d_sp_tiles = nullptr, *d_sp_tiles_mix = nullptr, *d_sp_tiles_pipe = nullptr;
   // the most dims of any copy item in a range [begin, end) of `items` (selects the
   // copy kernel built for at most 4 dims), computed on first use
