@@ -110,7 +110,7 @@ __device__ __forceinline__ void for_warp_range(const CopyJob *Js, int nj, int w0
 // copies straight into shared memory, all of an item's in flight at once.
 // Each warp takes one eighth of the item's elements in both phases.
 template <int ND, bool DENSE_SRC>
-__device__ __forceinline__ void stage_item(const CopyJob *Js, int nj, int total, const double *__restrict__ src,
+__device__ __forceinline__ void stage_item(const CopyJob *Js, int nj, int total, const double *src,
                                            double *__restrict__ dst, double *stage) {
   constexpr int kWarps = kThreads / 32;
   const int per_warp = (total + kWarps - 1) / kWarps;
@@ -159,7 +159,7 @@ __device__ __forceinline__ void stage_dispatch(bool dense_src, const CopyJob *Js
 // of 64 and fits five CTAs per SM instead of four.
 template <int MAXND>
 __device__ __forceinline__ void run_item(const CopyJob *__restrict__ jobs, const CopyItem &it,
-                                         const double *__restrict__ src, double *__restrict__ dst, CopyJob *Js,
+                                         const double *src, double *__restrict__ dst, CopyJob *Js,
                                          double *stage) {
   const int nj = it.njobs, total = it.total, nd = it.kind & 255, mode = it.kind >> 8;
   // the planner never makes other items, and the host never launches an item with
@@ -194,9 +194,9 @@ template <int MAXND>
 __global__ void __launch_bounds__(kThreads, MAXND <= 4 ? 5 : 4) copy_kernel(const CopyJob *__restrict__ jobs,
                                                                            const CopyItem *__restrict__ items,
                                                                            unsigned first,
-                                                                           const double *__restrict__ src,
+                                                                           const double *src,
                                                                            double *__restrict__ dst,
-                                                                           const double *__restrict__ src2,
+                                                                           const double *src2,
                                                                            double *__restrict__ dst2) {
   __shared__ CopyJob Js[kStageJobs];
   __shared__ double stage[kStageElems];
@@ -219,8 +219,8 @@ struct FlaggedGather {
 
 __global__ void __launch_bounds__(kThreads, 4) copy_flagged_kernel(const CopyJob *__restrict__ jobs,
                                                                    const SplitSector *__restrict__ sectors,
-                                                                   const int32_t *__restrict__ flagged,
-                                                                   const SplitRecord *__restrict__ rec,
+                                                                   const int32_t *flagged,
+                                                                   const SplitRecord *rec,
                                                                    FlaggedGather ga, FlaggedGather gb) {
   __shared__ CopyJob Js[kStageJobs];
   __shared__ double stage[kStageElems];
@@ -248,8 +248,8 @@ __global__ void __launch_bounds__(kThreads, 4) copy_flagged_kernel(const CopyJob
 // Zero fill of the flagged sectors' FP64 sector matrices (partially populated
 // operands) before their gathers.
 __global__ void __launch_bounds__(kThreads) zero_flagged_kernel(const SectorDev *__restrict__ sectors,
-                                                                const int32_t *__restrict__ flagged,
-                                                                const SplitRecord *__restrict__ rec, double *wa,
+                                                                const int32_t *flagged,
+                                                                const SplitRecord *rec, double *wa,
                                                                 double *wb, int zero_a, int zero_b) {
   after_previous_kernel();
   const int nflag = rec->nfallback;
@@ -278,7 +278,7 @@ constexpr int kTraceStage = 64;   // contributions kept in shared memory
 __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const TraceChunk *__restrict__ chunks,
                                                               const TraceOut *__restrict__ outs,
                                                               const TraceContrib *__restrict__ contribs,
-                                                              const double *__restrict__ src,
+                                                              const double *src,
                                                               double *__restrict__ dst) {
   __shared__ double part[kTraceThreads];
   __shared__ TraceContrib staged[kTraceStage];
@@ -372,7 +372,7 @@ __device__ __forceinline__ double plus_zero(double x) {
 // the GPU idle behind the largest blocks); chunks of 1024 take 9.8 us.
 __global__ void __launch_bounds__(256) cscatter_kernel(const CScatterJob *__restrict__ jobs,
                                                        const CScatterChunk *__restrict__ chunks,
-                                                       const double *__restrict__ P, double *__restrict__ C) {
+                                                       const double *P, double *__restrict__ C) {
   after_previous_kernel();
   const CScatterChunk ch = chunks[blockIdx.x];
   const CScatterJob J = jobs[ch.job];

@@ -43,7 +43,7 @@ __device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
 // Load one BK-slice of the A (or B) tile into registers: T x 16 elements, T/8 per
 // thread. kmajor: element (r, k) at base[r * ld + k]; else at base[k * ld + r].
 template <int T>
-__device__ __forceinline__ void load_tile(double (&v)[T / 8], const double *__restrict__ base, int ld, bool kmajor,
+__device__ __forceinline__ void load_tile(double (&v)[T / 8], const double *base, int ld, bool kmajor,
                                           int rows, int r0, int k0, int K) {
   const int t = threadIdx.x;
   if (kmajor) {
@@ -52,7 +52,7 @@ __device__ __forceinline__ void load_tile(double (&v)[T / 8], const double *__re
     for (int i = 0; i < T / 8; i++) {
       const int r = (t >> 4) + 8 * i;
       const int gr = r0 + r, gk = k0 + k;
-      v[i] = (gr < rows && gk < K) ? __ldg(base + (int64_t)gr * ld + gk) : 0.0;
+      v[i] = (gr < rows && gk < K) ? base[(int64_t)gr * ld + gk] : 0.0;
     }
   } else {
     const int r = t & (T - 1);
@@ -60,7 +60,7 @@ __device__ __forceinline__ void load_tile(double (&v)[T / 8], const double *__re
     for (int i = 0; i < T / 8; i++) {
       const int k = t / T + (kThreads / T) * i;
       const int gr = r0 + r, gk = k0 + k;
-      v[i] = (gr < rows && gk < K) ? __ldg(base + (int64_t)gk * ld + gr) : 0.0;
+      v[i] = (gr < rows && gk < K) ? base[(int64_t)gk * ld + gr] : 0.0;
     }
   }
 }
@@ -124,8 +124,8 @@ __device__ __forceinline__ void store_tile_out(const SectorDev &s, int sector, c
 // One T x T tile of C_q (T = 64, 32 or 16): four warps of (T/2) x (T/2), each a grid
 // of (T/16) x (T/16) DMMA 8x8 blocks.
 template <int T>
-__device__ __forceinline__ void gemm_tile(const SectorDev &s, const GemmTile &tl, const double *__restrict__ wa,
-                                          const double *__restrict__ wb, const OutView &out,
+__device__ __forceinline__ void gemm_tile(const SectorDev &s, const GemmTile &tl, const double *wa,
+                                          const double *wb, const OutView &out,
                                           double (*As)[BK][64 + PAD], double (*Bs)[BK][64 + PAD]) {
   constexpr int NB = T / 16;
   const int M = s.M, N = s.N, K = s.K;
@@ -193,8 +193,8 @@ __device__ __forceinline__ void gemm_tile(const SectorDev &s, const GemmTile &tl
 constexpr int kOuterK = 2;
 
 template <int COLS>
-__device__ __forceinline__ void outer_tile(const SectorDev &s, const GemmTile &tl, const double *__restrict__ wa,
-                                           const double *__restrict__ wb, const OutView &out, double (*As)[64],
+__device__ __forceinline__ void outer_tile(const SectorDev &s, const GemmTile &tl, const double *wa,
+                                           const double *wb, const OutView &out, double (*As)[64],
                                            OutRow *rows) {
   const int M = s.M, N = s.N, K = s.K, t = threadIdx.x;
   const int m0 = tl.mt * 64, n = tl.nt * COLS + (t & (COLS - 1));
@@ -211,7 +211,7 @@ __device__ __forceinline__ void outer_tile(const SectorDev &s, const GemmTile &t
   if (n < N) {
 #pragma unroll
     for (int k = 0; k < kOuterK; k++)
-      b[k] = k < K ? __ldg(wb + s.b_off + (s.b_kmajor ? (int64_t)n * K + k : (int64_t)k * N + n)) : 0.0;
+      b[k] = k < K ? wb[s.b_off + (s.b_kmajor ? (int64_t)n * K + k : (int64_t)k * N + n)] : 0.0;
     if (direct) col = out.cols[so.cols + n];
   }
   __syncthreads();
@@ -237,7 +237,7 @@ __device__ __forceinline__ void outer_tile(const SectorDev &s, const GemmTile &t
 // 67 MB) 38 us, 50 us as 64 x 64 tiles among the DMMA kernel's.
 __global__ void __launch_bounds__(256) gemm_outer_kernel(const SectorDev *__restrict__ sectors,
                                                          const GemmTile *__restrict__ tiles,
-                                                         const double *__restrict__ wa, const double *__restrict__ wb,
+                                                         const double *wa, const double *wb,
                                                          OutView out) {
   __shared__ double As[kOuterK][64];
   __shared__ OutRow rows[64];
@@ -249,8 +249,8 @@ __global__ void __launch_bounds__(256) gemm_outer_kernel(const SectorDev *__rest
 
 __global__ void __launch_bounds__(kThreads) gemm_fp64_kernel(const SectorDev *__restrict__ sectors,
                                                              const GemmTile *__restrict__ tiles,
-                                                             const double *__restrict__ wa,
-                                                             const double *__restrict__ wb, OutView out) {
+                                                             const double *wa,
+                                                             const double *wb, OutView out) {
   __shared__ double As[2][BK][64 + PAD];
   __shared__ double Bs[2][BK][64 + PAD];
   after_previous_kernel();
@@ -269,11 +269,11 @@ __global__ void __launch_bounds__(kThreads) gemm_fp64_kernel(const SectorDev *__
 // the check wrote on the device (tile_end: running tile counts per flagged
 // sector). With no flagged sector every CTA returns at once.
 __global__ void __launch_bounds__(kThreads) gemm_fp64_redo_kernel(const SectorDev *__restrict__ sectors,
-                                                                  const int32_t *__restrict__ flagged,
-                                                                  const int32_t *__restrict__ tile_end,
-                                                                  const SplitRecord *__restrict__ rec,
-                                                                  const double *__restrict__ wa,
-                                                                  const double *__restrict__ wb, OutView out) {
+                                                                  const int32_t *flagged,
+                                                                  const int32_t *tile_end,
+                                                                  const SplitRecord *rec,
+                                                                  const double *wa,
+                                                                  const double *wb, OutView out) {
   __shared__ double As[2][BK][64 + PAD];
   __shared__ double Bs[2][BK][64 + PAD];
   after_previous_kernel();

@@ -477,8 +477,8 @@ struct Cursor {
 template <int S, bool MIX>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     gemm_split_kernel(const SplitSector *__restrict__ sectors, const SplitTile *__restrict__ tiles, int ntiles,
-                      const uint8_t *__restrict__ sa, const uint8_t *__restrict__ sb, const int32_t *__restrict__ ea,
-                      const int32_t *__restrict__ eb, const int32_t *__restrict__ emax, float *__restrict__ normsq,
+                      const uint8_t *sa, const uint8_t *sb, const int32_t *ea,
+                      const int32_t *eb, const int32_t *emax, float *__restrict__ normsq,
                       OutView out, int *status) {
   using RG = Ring<S>;
   constexpr int kLeadP = 3 * kSliceBytes, kRestP = RG::kRest * kSliceBytes;   // P bytes of a slot
@@ -851,7 +851,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       // take, and nothing branches in between: 11,000 clocks for the CTA's 128 x 128
       // elements, against 16,000 with integers and a range check per element. The MMA
       // issuer waits for what exceeds the first chunk of the next tile.
-      const int pref = __ldg(emax + 2 * tl.sector + (swap ? 0 : 1)), qref = __ldg(emax + 2 * tl.sector + (swap ? 1 : 0));
+      const int pref = emax[2 * tl.sector + (swap ? 0 : 1)], qref = emax[2 * tl.sector + (swap ? 1 : 0)];
       const int64_t step = swap ? 1 : len;
       const int e0 = ep + qref - 2 * kExpBias - 40;
       uq = max(uq - qref, -4096);

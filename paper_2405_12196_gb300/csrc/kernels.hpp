@@ -34,6 +34,9 @@ cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, 
 #ifdef __CUDACC__
 // First in every kernel, before anything is read or written: waits until the stream's
 // previous kernels have finished and their writes are visible.
+// A kernel may have begun before its predecessor wrote what it reads, so only the plan's
+// tables, which no kernel writes, may be loaded as read-only for the kernel's lifetime (const
+// __restrict__ parameters, __ldg); data, workspace and records are loaded plainly.
 __device__ __forceinline__ void after_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 #endif
 

@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(kThreads) vdot_partial_kernel(const VdotChunk 
   }
 }
 
-__global__ void __launch_bounds__(kFinalThreads) vdot_final_kernel(const double *__restrict__ partials, int n,
+__global__ void __launch_bounds__(kFinalThreads) vdot_final_kernel(const double *partials, int n,
                                                                    double *out) {
   __shared__ double ws[kFinalThreads / 32];
   after_previous_kernel();

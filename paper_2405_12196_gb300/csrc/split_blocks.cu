@@ -171,7 +171,7 @@ struct Walk<1> {
 // else the rows).
 template <int ND, class S>
 __device__ __forceinline__ void load_units(S &sm, const SliceSeg &g, int u0, int u1, int lane,
-                                           const double *__restrict__ X) {
+                                           const double *X) {
   const int r0 = g.r0, nr = g.r1 - g.r0, k0 = g.k0, kc = g.k1 - g.k0;
   const double *base = X + g.boff;
   Walk<ND> w;
@@ -201,7 +201,7 @@ __device__ __forceinline__ void load_units(S &sm, const SliceSeg &g, int u0, int
 
 template <class S>
 __device__ __forceinline__ void load_units_any(S &sm, const SliceSeg &g, int u0, int u1, int lane,
-                                               const double *__restrict__ X) {
+                                               const double *X) {
   switch (g.rfast ? g.nk : g.nf) {
     case 0: load_units<0>(sm, g, u0, u1, lane, X); break;
     case 1: load_units<1>(sm, g, u0, u1, lane, X); break;
@@ -259,7 +259,7 @@ __device__ __forceinline__ void for_warp_share(const SliceItem &it, const SliceS
 // decomposed once per lane and part and stepped after that.
 template <class S>
 __device__ __forceinline__ void load_item(S &sm, const SliceItem &it, const SliceSeg *__restrict__ segs,
-                                          const double *__restrict__ X) {
+                                          const double *X) {
   const int tid = threadIdx.x, lane = tid & 31;
   if (!it.full) {   // the whole tile, pitch padding included, in 16-byte stores
     uint4 *z = reinterpret_cast<uint4 *>(&sm.tile[0][0]);
@@ -273,7 +273,7 @@ __device__ __forceinline__ void load_item(S &sm, const SliceItem &it, const Slic
 
 // The biased exponent of the double at p, from its upper word.
 __device__ __forceinline__ int biased_exp_at(const double *p) {
-  return (int)((__ldg(reinterpret_cast<const unsigned int *>(p) + 1) >> 20) & 0x7FF);
+  return (int)((reinterpret_cast<const unsigned int *>(p)[1] >> 20) & 0x7FF);
 }
 
 // Row maxima of the biased exponent over units [u0, u1) of a segment, combined into
@@ -288,7 +288,7 @@ __device__ __forceinline__ int biased_exp_at(const double *p) {
 // us. ND: the dims of the stepped side.
 template <int ND>
 __device__ __forceinline__ void rowmax_units(int *rmax, const SliceSeg &g, int u0, int u1, int lane,
-                                             const double *__restrict__ X) {
+                                             const double *X) {
   constexpr int kBatch = 8;
   const int r0 = g.r0, nr = g.r1 - g.r0, kc = g.k1 - g.k0;
   const double *base = X + g.boff;
@@ -347,8 +347,8 @@ template <bool BESIDE>
 __global__ void __launch_bounds__(kThreads, 8) split_rowmax_kernel(const SplitOperand *__restrict__ ops,
                                                                    const SliceItem *__restrict__ items, int nitems,
                                                                    const SliceSeg *__restrict__ segs,
-                                                                   const double *__restrict__ a,
-                                                                   const double *__restrict__ b,
+                                                                   const double *a,
+                                                                   const double *b,
                                                                    int32_t *__restrict__ ea, int32_t *__restrict__ eb,
                                                                    int32_t *__restrict__ emax) {
   __shared__ int rmax[kRowmaxItems][kItemRows];
@@ -406,8 +406,8 @@ __global__ void __launch_bounds__(kThreads, 8) split_rowmax_kernel(const SplitOp
 __global__ void __launch_bounds__(kThreads, 8) split_rowmax_tile_kernel(const SplitOperand *__restrict__ ops,
                                                                         const SliceItem *__restrict__ items,
                                                                         const SliceSeg *__restrict__ segs,
-                                                                        const double *__restrict__ a,
-                                                                        const double *__restrict__ b,
+                                                                        const double *a,
+                                                                        const double *b,
                                                                         int32_t *__restrict__ ea,
                                                                         int32_t *__restrict__ eb,
                                                                         int32_t *__restrict__ emax) {
@@ -448,10 +448,10 @@ template <int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) split_digits_kernel(const SplitOperand *__restrict__ ops,
                                                                       const SliceItem *__restrict__ items,
                                                                       const SliceSeg *__restrict__ segs,
-                                                                      const double *__restrict__ a,
-                                                                      const double *__restrict__ b,
-                                                                      const int32_t *__restrict__ ea,
-                                                                      const int32_t *__restrict__ eb,
+                                                                      const double *a,
+                                                                      const double *b,
+                                                                      const int32_t *ea,
+                                                                      const int32_t *eb,
                                                                       uint8_t *__restrict__ sa,
                                                                       uint8_t *__restrict__ sb, int s) {
   __shared__ Smem sm;

@@ -57,7 +57,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // This thread's share of the sum of 4^(e[i] - E) over rows [lo, hi).
-__device__ __forceinline__ double scale_sum(const int32_t *__restrict__ e, uint32_t lo, uint32_t hi, int E) {
+__device__ __forceinline__ double scale_sum(const int32_t *e, uint32_t lo, uint32_t hi, int E) {
   double s = 0.0;
   uint32_t i = lo + 4 * threadIdx.x;
 #pragma unroll 4
@@ -94,8 +94,8 @@ __device__ __forceinline__ int block_scan(int v, int *red, int *total) {
 
 __global__ void __launch_bounds__(kThreads) split_check_kernel(
     const SplitSector *__restrict__ sectors, int nsec, const SplitCheckChunk *__restrict__ chunks,
-    const int32_t *__restrict__ ea,
-    const int32_t *__restrict__ eb, const int32_t *__restrict__ emax, const float *__restrict__ normsq, double *secv,
+    const int32_t *ea,
+    const int32_t *eb, const int32_t *emax, const float *normsq, double *secv,
     int32_t *__restrict__ flagged, int32_t *__restrict__ tile_end, int32_t *__restrict__ item_end_a,
     int32_t *__restrict__ item_end_b, SplitRecord *rec, double eta_split, double eta_fp64, double rtol, int slices,
     int *status) {

@@ -38,8 +38,8 @@ namespace {
 // emax[op], the operand's largest (the reference scale of the accuracy check).
 __global__ void __launch_bounds__(256) split_exp_kernel(const SplitOperand *__restrict__ ops,
                                                         const SplitItem *__restrict__ items,
-                                                        const double *__restrict__ wa,
-                                                        const double *__restrict__ wb,
+                                                        const double *wa,
+                                                        const double *wb,
                                                         int32_t *__restrict__ ea, int32_t *__restrict__ eb,
                                                         int32_t *__restrict__ emax) {
   after_previous_kernel();
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(256) split_exp_kernel(const SplitOperand *__re
       const double *row = X + (int64_t)r * o.K;
       int m = 0;
 #pragma unroll 8
-      for (int k = k_lo + lane; k < k_hi; k += 32) m = max(m, biased_exp(__ldg(row + k)));
+      for (int k = k_lo + lane; k < k_hi; k += 32) m = max(m, biased_exp(row[k]));
 #pragma unroll
       for (int s = 16; s > 0; s >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, s));
       if (lane == 0) atomicMax(E + r, m);
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(256) split_exp_kernel(const SplitOperand *__re
     int m = 0;
     if (r < o.rows)
 #pragma unroll 4
-      for (int k = k_lo + half; k < k_hi; k += 2) m = max(m, biased_exp(__ldg(X + (int64_t)k * o.rows + r)));
+      for (int k = k_lo + half; k < k_hi; k += 2) m = max(m, biased_exp(X[(int64_t)k * o.rows + r]));
     red[half][rr] = m;
     mine = m;
     __syncthreads();
@@ -96,10 +96,10 @@ __global__ void __launch_bounds__(256) split_exp_kernel(const SplitOperand *__re
 // Slices: one 128 x 32 stage at a time through shared memory (raw FP64 bits).
 __global__ void __launch_bounds__(256, 6) split_slice_kernel(const SplitOperand *__restrict__ ops,
                                                           const SplitItem *__restrict__ items,
-                                                          const double *__restrict__ wa,
-                                                          const double *__restrict__ wb,
-                                                          const int32_t *__restrict__ ea,
-                                                          const int32_t *__restrict__ eb,
+                                                          const double *wa,
+                                                          const double *wb,
+                                                          const int32_t *ea,
+                                                          const int32_t *eb,
                                                           uint8_t *__restrict__ sa, uint8_t *__restrict__ sb,
                                                           int s) {
   __shared__ unsigned long long tile[kSplitBM][kSplitBK + 1];
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(256, 6) split_slice_kernel(const SplitOperand 
       for (int rr = warp; rr < kSplitBM; rr += 8) {
         const int r = r0 + rr, k = k0 + lane;
         double v = 0.0;
-        if (r < o.rows && k < o.K) v = __ldg(X + (int64_t)r * o.K + k);
+        if (r < o.rows && k < o.K) v = X[(int64_t)r * o.K + k];
         tile[rr][lane] = (unsigned long long)__double_as_longlong(v);
       }
     } else {
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(256, 6) split_slice_kernel(const SplitOperand 
         for (int q = 0; q < kSplitBM / 32; q++) {
           const int rr = q * 32 + lane, r = r0 + rr;
           double v = 0.0;
-          if (r < o.rows && k < o.K) v = __ldg(X + (int64_t)k * o.rows + r);
+          if (r < o.rows && k < o.K) v = X[(int64_t)k * o.rows + r];
           tile[rr][kk] = (unsigned long long)__double_as_longlong(v);
         }
       }

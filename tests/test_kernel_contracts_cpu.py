@@ -40,3 +40,29 @@ def test_split_gemm_outlasts_its_copies_and_mmas_after_an_abort():
     assert re.search(r"finish\(rest, nrest, RG::kRestStages", kernel)
     # the last commit arrives in both CTAs, which both wait for it
     assert "umma_commit(bar(kDone))" in kernel
+
+
+# what ytn_plan uploads and no kernel writes
+TABLES = {"CopyJob", "CopyItem", "SectorDev", "GemmTile", "TraceChunk", "TraceOut", "TraceContrib", "CScatterJob",
+          "CScatterChunk", "SplitOperand", "SplitItem", "SliceItem", "SliceSeg", "SplitSector", "SplitTile",
+          "SplitCheckChunk", "VdotChunk", "VdotPiece"}
+
+
+def test_only_the_plans_tables_are_read_as_constant():
+    """Kernels of a call start before their predecessor has finished and wait for it first:
+    what it wrote is not read-only for their lifetime."""
+    kernels = 0
+    for name in sorted(f for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh"))):
+        src = _source(name)
+        for m in re.finditer(r"const (\w+) \*__restrict__", src):
+            assert m.group(1) in TABLES, f"{name}: {m.group(0)}"
+        for m in re.finditer(r"__ldg\((\w+(?:\.\w+)?)", src):
+            assert m.group(1) in ("base", "out.base"), f"{name}: {src[m.start():m.start() + 60]}"
+        if "launch_chained(" not in src:
+            continue
+        for m in re.finditer(r"__global__", src):
+            body = _body(src, src.index(")", src.index("_kernel(", m.start())))
+            first = body.index("after_previous_kernel();")
+            assert not re.search(r"\w\[[^\]]*\](?!;)|->|=[^=]", re.sub(r"__shared__[^;]*;|constexpr[^;]*;|using[^;]*;|extern[^;]*;", "", body[:first])), name
+            kernels += 1
+    assert kernels >= 17
