@@ -1139,7 +1139,8 @@ static ytn_status run_move(ytn_plan_t *p, Kind k, const double *a, double *out, 
     return cuda_fail(e, "memset output");
   PhaseTimer t(p->ctx, YTN_PHASE_MOVE, st);
   if (k == Kind::Trace) {
-    if ((e = launch_trace(p->d_tr_chunks, (int64_t)p->tr_chunks.size(), p->d_tr_out, p->d_tr_contrib, a, out, st)) != cudaSuccess)
+    if ((e = launch_trace(p->d_tr_chunks, (int64_t)p->tr_chunks.size() - p->tr_flat, p->tr_flat, p->d_tr_out,
+                          p->d_tr_contrib, a, out, st)) != cudaSuccess)
       return cuda_fail(e, "trace");
     return YTN_OK;
   }

@@ -48,8 +48,9 @@ cudaError_t launch_copy(const CopyJob *jobs, const CopyItem *items, int64_t firs
                         double *dst, const double *src2, double *dst2, cudaStream_t stream,
                         int max_nd = kMaxCopyDims);
 
-// Trace: one CTA per chunk of an output block.
-cudaError_t launch_trace(const TraceChunk *chunks, int64_t nchunks, const TraceOut *outs,
+// Trace: one CTA per chunk of an output block, the first nsplit chunks with the terms shared
+// out over the threads, the nflat after them with a thread per element.
+cudaError_t launch_trace(const TraceChunk *chunks, int64_t nsplit, int64_t nflat, const TraceOut *outs,
                          const TraceContrib *contribs, const double *src, double *dst, cudaStream_t stream);
 
 // Scalar product <A, B> over the planned common elements (FP64, deterministic):

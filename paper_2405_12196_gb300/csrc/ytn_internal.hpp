@@ -114,8 +114,9 @@ struct GemmTile {
 };
 
 // Trace: one output block, fed by ncontrib contributing input blocks with nterms
-// diagonal elements in all; a CTA takes kTraceElems of its elements (TraceChunk).
-constexpr int kTraceElems = 32;
+// diagonal elements in all; a CTA takes kTraceElems of its elements (TraceChunk), or
+// kTraceFlatElems of a trace whose elements get a thread each.
+constexpr int kTraceElems = 32, kTraceFlatElems = 128;
 struct TraceChunk {
   int32_t out, e0;
 };
@@ -453,7 +454,8 @@ struct ytn_plan_s {
   std::vector<ytn::CScatterJob> cs_jobs;   // complex tensordot: the scatter-combine
   std::vector<ytn::CScatterChunk> cs_chunks;
   std::vector<ytn::TraceContrib> tr_contrib;
-  std::vector<ytn::TraceChunk> tr_chunks;
+  std::vector<ytn::TraceChunk> tr_chunks;   // the split ones first, then tr_flat flat ones
+  int64_t tr_flat = 0;
   std::vector<ytn::VdotPiece> vd_pieces;
   std::vector<ytn::VdotChunk> vd_chunks;
 
