@@ -742,9 +742,9 @@ ytn_status ytn_workspace_size(const ytn_plan_t *p, ytn_precision prec, double rt
 }
 
 // One contraction on the chosen path; arguments already checked and mapped. direct:
-// the GEMM may write C's blocks itself (C in device memory); complex products and
-// results in host memory go through the dense C_q and a scatter, whose writes run
-// along the blocks.
+// the GEMM may write C's blocks itself (C in device memory); complex products, results
+// in host memory and plans without the tables for it go through the dense C_q and a
+// scatter, whose writes run along the blocks.
 static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b, double *c, bool split, int slices,
                                  double rtol, void *workspace, cudaStream_t st, bool direct,
                                  bool fused_variant = false, bool narrow_tails = false, bool pipelined = false) {
@@ -754,7 +754,7 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
   double *wa = reinterpret_cast<double *>(ws + w.wa), *wb = reinterpret_cast<double *>(ws + w.wb),
          *wc = reinterpret_cast<double *>(ws + w.wc);
   cudaError_t e;
-  direct = direct && p->ca * p->cb == 1;
+  direct = direct && !p->out_sec.empty();
   const OutView out = direct ? OutView{p->d_out_sec, p->d_out_rows, p->d_out_cols, p->d_out_base, c}
                              : OutView{nullptr, nullptr, nullptr, nullptr, wc};
   // the fused split builds its slices straight from the blocks and gathers FP64

@@ -752,6 +752,13 @@ static void shard_sectors(ytn_plan_t *p, const Tensor &A, const Tensor &B,
   p->flops = kept * p->ca * p->cb;
 }
 
+// Whether the GEMMs get tables of C's rows, columns and blocks (`table` bytes, kept on the
+// device as long as the plan): up to 1 MiB, or a sixteenth of what C's data and the scatter's
+// jobs take (`held`). Wide products need far less (the D = 20 environment 0.2%); a product
+// with a thin side, a gate's, would keep a table half the size of its operand, and
+// goes through the dense C_q and the scatter.
+static bool out_tables_fit(int64_t table, int64_t held) { return table <= std::max<int64_t>(1 << 20, held / 16); }
+
 ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int naxes,
                           const int *axa_in, const int *axb_in, std::string &err) {
   if (A.nsym != B.nsym || std::memcmp(A.mod, B.mod, sizeof(A.mod)) != 0) {
@@ -1068,8 +1075,7 @@ ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int n
 
   // Output blocks: (I, J) exists when some x has both A(I, x) and B(x, J).
   std::vector<OutBlock> outb;
-  struct Src { int64_t sector; int64_t roff, coff; int64_t nI, nJ; int64_t a_blk, b_blk; int64_t base; };
-  const bool direct = ca * cb == 1;   // the GEMMs write C's blocks themselves
+  struct Src { int64_t sector; int64_t roff, coff; int64_t nI, nJ; int64_t a_blk, b_blk; int64_t at; };
   p->out_sec.clear();
   p->out_rows.clear();
   p->out_cols.clear();
@@ -1096,23 +1102,6 @@ ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int n
         v[xi / 64] |= 1ull << (xi % 64);
       }
     }
-    int64_t base = 0;   // this sector's table of block offsets, filled once C is laid out
-    if (direct) {
-      base = (int64_t)p->out_base.size();
-      p->out_sec.push_back({(int64_t)p->out_rows.size(), (int64_t)p->out_cols.size(), base, (int32_t)sb.cols.size(), 0});
-      p->out_base.resize(p->out_base.size() + sb.rows.size() * sb.cols.size(), -1);
-      int32_t blk = 0;
-      for (auto &r : sb.rows) {
-        for (int64_t i = 0; i < r.second.first; i++) p->out_rows.push_back({blk, (int32_t)i});
-        blk++;
-      }
-      blk = 0;
-      for (auto &c : sb.cols) {
-        for (int64_t j = 0; j < c.second.first; j++)
-          p->out_cols.push_back({blk, (int32_t)j, (int32_t)c.second.first, 0});
-        blk++;
-      }
-    }
     int64_t at = -1;   // (row block, column block) in the sector's table
     for (auto &r : sb.rows) {
       const auto &rv = rowx[r.first];
@@ -1130,15 +1119,40 @@ ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int n
         ob.id = (int64_t)srcs.size();
         outb.push_back(ob);
         srcs.push_back({(int64_t)si, g.row_off.at(r.first), g.col_off.at(c.first), r.second.first,
-                        c.second.first, r.second.second, c.second.second, base + at});
+                        c.second.first, r.second.second, c.second.second, at});
       }
     }
   }
   std::vector<int64_t> off_of_id;
   finalize_out(C, outb, off_of_id);
-  if (direct)
-    for (size_t id = 0; id < srcs.size(); id++) p->out_base[srcs[id].base] = off_of_id[id];
-  // Scatter C (into host memory; else the GEMMs write it): block (I, J) = C_q[row_off(I) + i, col_off(J) + j], row-major per leg.
+  // The tables by which the GEMMs write C's blocks themselves, when they stay small beside
+  // what the plan and C hold in any case.
+  int64_t table = 0, held = 0;
+  for (size_t si = 0; si < geo.size(); si++)
+    table += (int64_t)sizeof(OutRow) * geo[si].M + (int64_t)sizeof(OutCol) * geo[si].N +
+             (int64_t)sizeof(int64_t) * (int64_t)(sbs[si]->rows.size() * sbs[si]->cols.size());
+  for (const Src &sr : srcs) held += 8 * sr.nI * sr.nJ + (int64_t)sizeof(CopyJob);
+  if (ca * cb == 1 && out_tables_fit(table, held)) {
+    for (size_t si = 0; si < geo.size(); si++) {
+      const SB &sb = *sbs[si];
+      p->out_sec.push_back({(int64_t)p->out_rows.size(), (int64_t)p->out_cols.size(), (int64_t)p->out_base.size(),
+                            (int32_t)sb.cols.size(), 0});
+      p->out_base.resize(p->out_base.size() + sb.rows.size() * sb.cols.size(), -1);
+      int32_t blk = 0;
+      for (auto &r : sb.rows) {
+        for (int64_t i = 0; i < r.second.first; i++) p->out_rows.push_back({blk, (int32_t)i});
+        blk++;
+      }
+      blk = 0;
+      for (auto &c : sb.cols) {
+        for (int64_t j = 0; j < c.second.first; j++)
+          p->out_cols.push_back({blk, (int32_t)j, (int32_t)c.second.first, 0});
+        blk++;
+      }
+    }
+    for (size_t id = 0; id < srcs.size(); id++) p->out_base[p->out_sec[srcs[id].sector].base + srcs[id].at] = off_of_id[id];
+  }
+  // Scatter C (complex, in host memory, or without those tables): block (I, J) = C_q[row_off(I) + i, col_off(J) + j], row-major per leg.
   p->cs_jobs.clear();
   p->cs_chunks.clear();
   for (size_t id = 0; id < srcs.size() && ca * cb > 1; id++) {

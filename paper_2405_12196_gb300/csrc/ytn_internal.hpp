@@ -97,7 +97,8 @@ struct SectorOut {
 };
 // The tables on the device and the destination: C's data (tables set), or with null
 // tables the dense sector matrices of the workspace (row-major at SectorDev::c_off;
-// complex products and results in host memory, scattered by the copy kernels).
+// complex products, results in host memory and plans whose tables would be large,
+// scattered by the copy kernels).
 struct OutView {
   const SectorOut *sec;
   const OutRow *rows;
@@ -459,7 +460,8 @@ struct ytn_plan_s {
   std::vector<ytn::VdotPiece> vd_pieces;
   std::vector<ytn::VdotChunk> vd_chunks;
 
-  // real tensordot: C's blocks as the GEMMs address them (empty for complex products)
+  // real tensordot: C's blocks as the GEMMs address them (empty for complex products, and
+  // where the tables would be large: out_tables_fit)
   std::vector<ytn::SectorOut> out_sec;
   std::vector<ytn::OutRow> out_rows;
   std::vector<ytn::OutCol> out_cols;
