@@ -585,9 +585,9 @@ def measure_contraction(args, ytn, ctx, dev, cfg, world, rank, local, prec, step
     # ---- headline precision: device-resident steps
     head = measure(prec, steps, warmup, clocks=True)
     ph = phases(head)
-    # the gathers of A and B are one launch (timed as gather_a); the fused split path reads
-    # their blocks in its slicing kernels (the split phase) instead, and the GEMMs write C's
-    # blocks themselves unless C is complex (or in host memory): then a scatter does
+    # the gathers of A and B are one launch each while phases are timed; the fused split
+    # path reads their blocks in its slicing kernels (the split phase) instead, and the GEMMs
+    # write C's blocks themselves unless C is complex (or in host memory): then a scatter does
     moved_bytes = 16.0 * (((plan.info["moved_elems"] - plan.info["out_size"]) if "gather_a" in ph else 0)
                           + (plan.info["out_size"] if "scatter" in ph else 0))
     mover_ms = sum(ph[k]["ms_per_call"] for k in ("gather_a", "gather_b", "scatter") if k in ph)

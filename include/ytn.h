@@ -666,9 +666,13 @@ void ytn_server_destroy(ytn_server_t *server);
  * phase into *out and clears the record. Phases: */
 enum {
   YTN_PHASE_GATHER_A = 0,   /* blocks of A -> sector matrices                 */
-  YTN_PHASE_GATHER_B = 1,   /* blocks of B -> sector matrices                 */
-  YTN_PHASE_GEMM = 2,       /* grouped GEMM (FP64 or split-precision)         */
-  YTN_PHASE_SCATTER = 3,    /* sector matrices -> blocks of C                 */
+  YTN_PHASE_GATHER_B = 1,   /* blocks of B -> sector matrices (one launch with
+                               A's while phases are not timed)                */
+  YTN_PHASE_GEMM = 2,       /* grouped GEMM (FP64 or split-precision), most often
+                               with the blocks of C as its output             */
+  YTN_PHASE_SCATTER = 3,    /* sector matrices -> blocks of C, where the GEMM does
+                               not write them: complex products, C in host memory
+                               or over an operand, products with a long thin side */
   YTN_PHASE_SPLIT = 4,      /* FP64 -> BF16 slices (split path)               */
   YTN_PHASE_MOVE = 5,       /* fuse / unfuse / trace                          */
   YTN_PHASE_REDUCE = 6,     /* scalar products                                */

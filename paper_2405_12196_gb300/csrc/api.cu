@@ -765,10 +765,17 @@ static ytn_status exec_tensordot(ytn_plan_t *p, const double *a, const double *b
       return cuda_fail(e, "memset A workspace");
     if (p->zero_b && (e = cudaMemsetAsync(wb, 0, (size_t)p->b_elems * 8, st)) != cudaSuccess)
       return cuda_fail(e, "memset B workspace");
+    // both operands' items follow one another in the table: one launch, or two while the
+    // phases are timed
+    const bool apart = p->ctx->prof;
     {
-      // both operands' items follow one another in the table: one launch
       PhaseTimer t(p->ctx, YTN_PHASE_GATHER_A, st);
-      e = copy_range(p, p->items_a_begin, p->items_b_end, a, wa, st, p->items_a_end - p->items_a_begin, b, wb);
+      e = copy_range(p, p->items_a_begin, apart ? p->items_a_end : p->items_b_end, a, wa, st,
+                     p->items_a_end - p->items_a_begin, b, wb);
+    }
+    if (e == cudaSuccess && apart) {
+      PhaseTimer t(p->ctx, YTN_PHASE_GATHER_B, st);
+      e = copy_range(p, p->items_b_begin, p->items_b_end, b, wb, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "gather the operands");
   }
