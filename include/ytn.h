@@ -405,21 +405,24 @@ ytn_status ytn_workspace_size_staged(const ytn_plan_t *plan, ytn_precision prec,
  * from page-locked host memory (no staging workspace) always take the staged
  * variant, whose gathers read every block linearly over the host link.
  * A large plan (sectors enough for at least two groups of about an eighth of the
- * useful FLOPs and two waves of 128-wide tiles each) also times the fused variant
+ * useful FLOPs and two waves of GEMM tiles each) also times the fused variant
  * pipelined with the GEMM: the sectors in groups, each group's slices built on
  * the lowest-priority stream of the context while the previous group's GEMM runs
- * on its highest-priority stream (a slicing CTA shares each SM with a GEMM CTA),
- * forked from and joined to the caller's stream; one pipelined call is enqueued
+ * on its highest-priority stream (with four slices a slicing CTA shares each SM
+ * with a GEMM CTA; with more the GEMM's shared memory leaves no room, and slicing
+ * runs on the SMs that a GEMM does not fill), forked from and joined to the
+ * caller's stream; one pipelined call is enqueued
  * at a time per context, and a call on a stream being captured into a graph does
  * not pipeline. res->split_variant reports the variant used.
- * Likewise the split GEMM's tile list: 128 x 128 tiles, or the same with a
- * 128 x 64 last column tile for every sector whose N ends in the first half of a
- * 128-wide tile (half of that tile's padded products saved); the first split call
+ * Likewise the split GEMM's tile list: tiles of 128 rows x 256 columns of a sector's
+ * product, one per pair of CTAs, or for every sector whose N ends in the first half
+ * of a 128-wide tile 256 rows x 128 columns with a last column tile 64 wide (half
+ * of that tile's padded products saved); the first split call
  * times both when the plan has such sectors (all 128 wide under graph capture);
  * res->narrow_tiles reports the choice.
  * On the split path the call also checks its own accuracy on the device (see
  * ytn_error_report): sectors whose data-aware estimate exceeds rtol are
- * recomputed on the FP64 path before C is written, and when even that leaves
+ * recomputed on the FP64 path, over what the split GEMM wrote, and when even that leaves
  * the estimate above rtol the next ytn_sync on the context returns
  * YTN_E_TOLERANCE. The slice count comes from an a-priori forecast for typical
  * data (s = 5 at rtol 1e-10, s = 6 down to about 1.5e-11); the device check makes

@@ -231,14 +231,14 @@ __device__ __forceinline__ void outer_tile(const SectorDev &s, const GemmTile &t
   }
 }
 
-// Plans of such sectors only (tiles of 64 x 128, 128 the tile's size): small shared
-// memory, so that eight CTAs per SM hide the loads at a tile's start. Bound by the FP64
-// multiplications, 16 clocks a warp and SM; the Z2 D = 8 double layer (8.4e6 elements,
-// 67 MB) 38 us, 50 us as 64 x 64 tiles among the DMMA kernel's.
+// Plans of such sectors only (tiles of 64 x 128, 128 the tile's size). The Z2 D = 8 double
+// layer (8.4e6 elements, 67 MB) takes 38 us, 50 us as 64 x 64 tiles among the DMMA kernel's.
+// Neither the FP64 multiplications (16 clocks a warp and SM: 14 us) nor the stores (10 us at
+// the copy peak) bound it: 48 registers let five CTAs share an SM, so that its 1024 CTAs
+// are 1.35 waves, and each begins with a chain of loads (tile, sector, tables, operands).
 __global__ void __launch_bounds__(256) gemm_outer_kernel(const SectorDev *__restrict__ sectors,
                                                          const GemmTile *__restrict__ tiles,
-                                                         const double *wa, const double *wb,
-                                                         OutView out) {
+                                                         const double *wa, const double *wb, OutView out) {
   __shared__ double As[kOuterK][64];
   __shared__ OutRow rows[64];
   after_previous_kernel();

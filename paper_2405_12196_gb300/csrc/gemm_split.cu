@@ -47,9 +47,11 @@
 //              (peer CTA) relays its "stage loaded" signals to the leader;
 //   warps 2-17 (both CTAs) epilogue: chunk drains and the FP64 output (four warps per
 //              32-lane quarter of tensor memory, 32 columns each; warp 2 also
-//              allocates and frees tensor memory), which keeps the 64-bit
-//              accumulators in registers under the 96-register budget of a
-//              576-thread CTA, and writes C's blocks (OutView) or the dense C_q.
+//              allocates and frees tensor memory), whose 32 64-bit accumulators per
+//              lane take most of the 96 registers that a 576-thread CTA leaves a thread
+//              (the output, which needs tables and places beside them, spills 108 bytes
+//              of stores and 172 of loads; with 64-wide tails 200 and 384), and writes
+//              C's blocks (OutView) or the dense C_q.
 // Bound by the tensor cores, and on large contractions by power. An MMA takes 64 clocks
 // per SM, a stage of five slices 1920. On the D = 20 environment (15 slice products of
 // 1.86e12 FLOPs) a stage took 2940 clocks with one CTA per 128 x 128 tile (18.1 ms, and
