@@ -141,19 +141,26 @@ __global__ void __launch_bounds__(kThreads) split_check_kernel(
 
   // the sums of sectors of several chunks into their first chunk's place, a warp per sector
   if (!single) {
-    for (int s = warp; s < nsec; s += kThreads / 32) {
-      const int c0 = sectors[s].chk0, c1 = sectors[s].chk1;
-      if (c1 - c0 < 2) continue;
-      double se = 0.0, sf = 0.0;
-      for (int c = c0 + lane; c < c1; c += 32) {
-        se += __ldcg(secv + 2 * c);
-        sf += __ldcg(secv + 2 * c + 1);
+    for (int base = 32 * warp; base < nsec; base += kThreads) {
+      int c0 = 0, n = 0;
+      if (base + lane < nsec) {
+        c0 = sectors[base + lane].chk0;
+        n = sectors[base + lane].chk1 - c0;
       }
-      se = warp_sum(se);
-      sf = warp_sum(sf);
-      if (lane == 0) {
-        __stcg(secv + 2 * c0, se);
-        __stcg(secv + 2 * c0 + 1, sf);
+      for (uint32_t many = __ballot_sync(0xffffffffu, n > 1); many; many &= many - 1) {
+        const int b = __ffs(many) - 1;
+        const int from = __shfl_sync(0xffffffffu, c0, b), to = from + __shfl_sync(0xffffffffu, n, b);
+        double se = 0.0, sf = 0.0;
+        for (int c = from + lane; c < to; c += 32) {
+          se += __ldcg(secv + 2 * c);
+          sf += __ldcg(secv + 2 * c + 1);
+        }
+        se = warp_sum(se);
+        sf = warp_sum(sf);
+        if (lane == 0) {
+          __stcg(secv + 2 * from, se);
+          __stcg(secv + 2 * from + 1, sf);
+        }
       }
     }
     __syncthreads();
