@@ -55,6 +55,17 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// The warp's sums of a (in lanes 0..15) and b (in lanes 16..31), with half the additions of
+// two sums: an FP64 addition takes a warp 16 clocks of the SM's FP64 pipe.
+__device__ __forceinline__ double warp_sum2(double a, double b) {
+  const bool upper = (threadIdx.x & 16) != 0;
+  double v = upper ? b : a;
+  v += __shfl_xor_sync(0xffffffffu, upper ? a : b, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // This thread's share of the sum of 4^(e[i] - E) over rows [lo, hi).
 __device__ __forceinline__ double scale_sum(const int32_t *e, uint32_t lo, uint32_t hi, int E) {
   double s = 0.0;
@@ -114,12 +125,8 @@ __global__ void __launch_bounds__(kThreads) split_check_kernel(
     if (lo < sc.M) se = scale_sum(ea + sc.ea_off, lo, min((int64_t)sc.M, hi), emax[2 * q]);
     if (hi > mb && lo - mb < sc.N)
       sf = scale_sum(eb + sc.eb_off, max((int64_t)0, lo - mb), min((int64_t)sc.N, hi - mb), emax[2 * q + 1]);
-    se = warp_sum(se);
-    sf = warp_sum(sf);
-    if (lane == 0) {
-      dred[0][warp] = se;
-      dred[1][warp] = sf;
-    }
+    const double v = warp_sum2(se, sf);
+    if ((lane & 15) == 0) dred[lane >> 4][warp] = v;
     __syncthreads();
   }
   // the last CTA to get here sees every sector's sums (one thread writes and fences: all
@@ -155,12 +162,8 @@ __global__ void __launch_bounds__(kThreads) split_check_kernel(
           se += __ldcg(secv + 2 * c);
           sf += __ldcg(secv + 2 * c + 1);
         }
-        se = warp_sum(se);
-        sf = warp_sum(sf);
-        if (lane == 0) {
-          __stcg(secv + 2 * from, se);
-          __stcg(secv + 2 * from + 1, sf);
-        }
+        const double v = warp_sum2(se, sf);
+        if ((lane & 15) == 0) __stcg(secv + 2 * from + (lane >> 4), v);
       }
     }
     __syncthreads();
@@ -225,11 +228,13 @@ __global__ void __launch_bounds__(kThreads) split_check_kernel(
     nia += total_ia;
     nib += total_ib;
   }
-  norm = warp_sum(norm);
-  err_split = warp_sum(err_split);
-  err_after = warp_sum(err_after);
+  if (32 * warp < nsec) {   // the others looked at no sector
+    norm = warp_sum(norm);
+    err_split = warp_sum(err_split);
+    err_after = warp_sum(err_after);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) worst = fmax(worst, __shfl_xor_sync(0xffffffffu, worst, o));
+    for (int o = 16; o > 0; o >>= 1) worst = fmax(worst, __shfl_xor_sync(0xffffffffu, worst, o));
+  }
   if (lane == 0) {
     dred[0][warp] = norm;
     dred[1][warp] = err_split;
