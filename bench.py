@@ -495,7 +495,7 @@ def strong_value(total_flops, steps, seconds):
 # ------------------------------------------------------------------ our arm
 
 def measure_contraction(args, ytn, ctx, dev, cfg, world, rank, local, prec, steps, warmup, e2e_steps, fp64_steps,
-                        nfly=3):
+                        nfly=3, workload=None):
     """Time one contraction (this rank's part of it when world > 1) through the C ABI:
     the headline precision on device-resident data (CUDA events on the launching stream,
     clocks sampled meanwhile), the FP64 path beside it, and end to end with page-locked
@@ -574,7 +574,7 @@ def measure_contraction(args, ytn, ctx, dev, cfg, world, rank, local, prec, step
                     f"(s(s+1)/2 = {s_ * (s_ + 1) // 2} per useful FLOP, s = {s_} slices)")
         achieved = kflops / (kernel_ms * 1e-3) / 1e12 if kernel_ms > 0 else None
         return {"bound": "tensor", "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": (achieved / peak) if achieved else None, "traffic": read_traffic(kernel, args.workload),
+                "frac": (achieved / peak) if achieved else None, "traffic": read_traffic(kernel, workload or args.workload),
                 "kernel_ms": kernel_ms,
                 "effective_fp64_tflops": flops / (kernel_ms * 1e-3) / 1e12 if kernel_ms else None,
                 "peak_source": note}
@@ -845,7 +845,7 @@ def extra_cfg5b(args, ytn, ctx, dev, prec):
     to 11388^3), a few steps: value, roofline and e2e on the same clock as the headline."""
     cfg = make_workload("cfg5b", 0)
     m = measure_contraction(args, ytn, ctx, dev, cfg, 1, 0, 0, prec, args.extra_steps, 3, args.extra_steps, 0,
-                            nfly=2)
+                            nfly=2, workload="cfg5b")
     out = {"workload": WORKLOAD_DESC["cfg5b"], "useful_flops_per_step": m["total_flops"], "value": m["value"],
            "unit": "TFLOP/s", "steps": args.extra_steps, "warmup": 3, "ms_per_step": m["ms_per_step"],
            "sectors": m["plan"].info["nsectors"],

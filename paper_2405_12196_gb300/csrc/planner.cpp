@@ -756,7 +756,9 @@ static void shard_sectors(ytn_plan_t *p, const Tensor &A, const Tensor &B,
 // device as long as the plan): up to 1 MiB, or a sixteenth of what C's data and the scatter's
 // jobs take (`held`). Wide products need far less (the D = 20 environment 0.2%); a product
 // with a thin side, a gate's, would keep a table half the size of its operand, and
-// goes through the dense C_q and the scatter.
+// goes through the dense C_q and the scatter (2e6 x 4 x 4: plan 14.7 MB and 9.1 ms instead of
+// 31.5 MB and 16.6 ms, FP64 call 474 us instead of 584; twenty such shapes 19% faster to 8%
+// slower than with tables).
 static bool out_tables_fit(int64_t table, int64_t held) { return table <= std::max<int64_t>(1 << 20, held / 16); }
 
 ytn_status plan_tensordot(ytn_plan_t *p, const Tensor &A, const Tensor &B, int naxes,
